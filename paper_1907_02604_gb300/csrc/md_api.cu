@@ -15,6 +15,7 @@
 
 #include "md_adjoint.h"
 #include "md_internal.h"
+#include "md_krylov.h"
 #include "md_lanczos.h"
 #include "md_solver.h"
 
@@ -117,7 +118,7 @@ void free_ham(Ham& H) {
     }
     void* ptrs[] = {H.V, H.V32, H.atom_xyz, H.atom_depth, H.atom_sigma, H.proj_i0, H.proj_len,
                     H.proj_d, H.proj_g, H.proj_d32, H.proj_g32, H.proj_C, H.proj_absum,
-                    H.proj_C32, H.proj_rows, H.pl_ptr, H.pl_atom, H.pl_val32, H.pl_val64,
+                    H.proj_C32, H.proj_rows, H.pl_ptr, H.pl_atom, H.pl_val32, H.pl_val64, H.proj_fx, H.proj_fxc,
                     H.scratch, H.lz_buf};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -236,6 +237,318 @@ md_status upload_poles(const md_poles* poles, double2** d_z, double2** d_w, cuda
 }  // namespace
 }  // namespace md
 
+namespace md {
+namespace {
+
+// ---------------------------------------------------------------------------
+// Node-shared Krylov solves (md_krylov.cu): shapes and launches.
+// ---------------------------------------------------------------------------
+
+constexpr int kKryClasses = 12;   // region-size classes of one batch, launched side by side
+constexpr int kKryStreams = 4;    // the caller's stream and the three of KrySide
+
+}  // namespace
+
+struct KryClass {
+    int csz, block, grid;
+    size_t smem;
+    KrylovParams P;
+};
+
+// Side streams of a launch of several classes.
+struct KrySide {
+    cudaStream_t s[3] = {};
+    cudaEvent_t fork = nullptr, join[3] = {};
+};
+
+namespace {
+
+// Power of two at least twice ||H_R - shift|| (Gershgorin bounds, projector
+// terms counted apart), so that the scaled operator has norm < 1/2 and every
+// fixed-point sum of md_krylov.cu stays in range; 0 if there is none.
+double kry_scale(const Ham& H) {
+    const double e = H.nonlocal && H.n_atoms > 0 ? std::fabs(H.e_s) + 3.0 * std::fabs(H.e_p) : 0.0;
+    const double b = std::max(std::fabs(H.emax - H.diag), std::fabs(H.emin - H.diag)) + H.pl_max * e;
+    const double need = std::max(2.0 * b, 32.0 * e);
+    if (!H.bounds_valid || !(need > 1e-30 && need < 1e30)) return 0.0;
+    return std::exp2(std::ceil(std::log2(need)) + 0.0);
+}
+
+void kry_operator(KrylovParams& P, const Ham& H, double scale) {
+    P.scale = scale;
+    P.shift = H.diag;
+    for (int d = 0; d < 3; ++d)
+        for (int o = 0; o < kKryMaxQ; ++o) {
+            const long long x = o < H.q ? std::llrint(std::ldexp(H.coef[d][o] / scale, 62)) : 0;
+            const long long hi = (x + (1LL << 30)) >> 31;
+            P.wh[d][o] = (int)hi;
+            P.wl[d][o] = (int)(x - (hi << 31));
+        }
+}
+
+struct KryShape {
+    int csz = 0, block = 0, per_sm = 1, clusters = 0, depth = 0;
+    size_t smem = 0;
+    bool spill = false;  // projector tables do not fit in shared memory
+    double time = 0.0;   // model of one Krylov step, cycles
+};
+
+// Clusters of c CTAs that fit the device with one CTA per SM.
+int kry_clusters_alone(int c) {
+    static std::mutex mu;
+    static int n[16][9] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> g(mu);
+    int& v = n[dev & 15][c];
+    if (v == 0) v = kry_max_clusters(4, 0, c, kry_max_threads() + 32, 160 * 1024);
+    return v;
+}
+
+// Shape of c CTAs for regions of at most m0 x m1 x m2 points; csz = 0 if the
+// slabs do not fit.
+KryShape kry_shape(const Ham& H, int m0, int m1, int m2, int c, int dev) {
+    KryShape s;
+    const bool nl = H.nonlocal && H.n_atoms > 0;
+    int optin = 0;
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    const size_t budget = (size_t)optin - kry_static_smem_bytes(nl);
+    s.depth = (m2 + c - 1) / c;
+    const long long ncol = (long long)m0 * m1;
+    if (c > m2 || s.depth > kKryMaxDepth) return s;
+    if (nl && ncol * s.depth * H.pl_max >= 65535) return s;   // 16-bit row ids
+    const size_t u = kry_u_bytes(H.q, m0, m1, s.depth);
+    // projector tables: fixed parts, and what the average density suggests for
+    // row factors and x tables (they fall back to device memory if short)
+    size_t tables = 0;
+    if (nl) {
+        const double reach[3] = {m0 + 2 * H.proj_rc / H.h[0], m1 + 2 * H.proj_rc / H.h[1],
+                                 s.depth + 2 * H.proj_rc / H.h[2]};
+        const double per_pt = (double)H.n_atoms / H.N;
+        const double local = std::min<double>(per_pt * reach[0] * reach[1] * (m2 + 2 * H.proj_rc / H.h[2]),
+                                              std::min<double>(H.n_atoms, kMaxLocalProjAtoms));
+        const double here = std::min(local, per_pt * reach[0] * reach[1] * reach[2]);
+        const double rows = here * 3.2 * H.proj_rc * H.proj_rc / (H.h[1] * H.h[2]) * m1 / reach[1] * s.depth / reach[2];
+        tables = (size_t)(kry_max_threads() * 32 + 1024 + local * 96);
+        if (u + kry_max_threads() * 32 + 1024 > budget) return s;
+        s.spill = u + tables + (size_t)(1.15 * (rows + here * 2.0 * H.proj_rc / H.h[0]) * 16) > budget;
+    } else if (u > budget) {
+        return s;
+    }
+    s.smem = nl ? budget : u;
+    // the fewest warps within 3 % of the best split of the slab's pairs
+    const long long tasks = (ncol / m0 * ((m0 + 1) / 2) * s.depth + 31) / 32;
+    double best = 0.0;
+    int nw = 0;
+    for (int w = kry_max_threads() / 32; w >= 2; --w) {
+        const double cost = (double)((tasks + w - 1) / w) * (w + 12);   // a step's latency, and its issue slots
+        if (nw == 0 || cost < 1.03 * best) {
+            best = nw == 0 ? cost : std::min(best, cost);
+            nw = w;
+        }
+    }
+    s.block = 32 * nw + 32;
+    s.per_sm = std::max(1, std::min({(int)(232448 / (s.smem + kry_static_smem_bytes(nl) + 1024)), 2048 / s.block,
+                                     24 / (s.block / 32)}));
+    s.clusters = kry_clusters_alone(c) * s.per_sm;
+    // a step, measured in cycles: 8 a warp's 32 pairs and warp in flight (11 with
+    // projectors), 3,000 a plane for the projections, the exchanges
+    s.time = s.per_sm * best * (nl ? (s.spill ? 22.0 : 11.0) : 8.0) +
+             (nl ? 18000.0 + s.per_sm * 3000.0 * s.depth * (m0 * m1 / 1089.0) : 8000.0);
+    s.csz = c;
+    return s;
+}
+
+// Size classes of the batch and a shape for each; false if some region does
+// not fit.  order: nodes, largest class first; first[k]..first[k+1] is class k.
+bool kry_classes(const Ham& H, const Regions& R, std::vector<int>& order, std::vector<int>& first,
+                 std::vector<KryShape>& shapes, std::vector<NodeDesc>& dims) {
+    const int nn = (int)R.desc.size();
+    if (H.q > kKryMaxQ || R.any_ring || nn == 0) return false;
+    if (H.nonlocal && H.n_atoms > 0 && !H.proj_fx_ok) return false;
+    order.resize(nn);
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return R.points[a] > R.points[b]; });
+    std::vector<long long> sizes;
+    for (int j : order)
+        if (sizes.empty() || sizes.back() != R.points[j]) sizes.push_back(R.points[j]);
+    const int per = ((int)sizes.size() + kKryClasses - 1) / kKryClasses;   // sizes a class
+    first.clear();
+    size_t si = 0;
+    for (int i = 0; i < nn; ++i) {
+        if (R.points[order[i]] != sizes[si]) ++si;
+        if (i == 0 || (si % per == 0 && R.points[order[i - 1]] != R.points[order[i]])) first.push_back(i);
+    }
+    first.push_back(nn);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int nc = (int)first.size() - 1;
+    std::vector<std::vector<KryShape>> cand(nc);
+    dims.assign(nc, NodeDesc{});
+    for (int k = 0; k < nc; ++k) {
+        for (int i = first[k]; i < first[k + 1]; ++i)
+            for (int d = 0; d < 3; ++d) dims[k].dims[d] = std::max(dims[k].dims[d], R.desc[order[i]].dims[d]);
+        for (int c = 1; c <= 8; ++c) {
+            KryShape s = kry_shape(H, dims[k].dims[0], dims[k].dims[1], dims[k].dims[2], c, dev);
+            if (s.csz > 0 && s.clusters > 0) cand[k].push_back(s);
+        }
+        if (cand[k].empty()) return false;
+    }
+    // Krylov steps grow about linearly with the region's extent.  One class:
+    // the shape with the shortest makespan.  Several share the device: each
+    // takes the shape with the least SM time, then those whose nodes alone
+    // would outlast the rest move to more CTAs a node.
+    shapes.assign(nc, KryShape{});
+    if (nc == 1) {
+        double best = 0.0;
+        for (const KryShape& s : cand[0]) {
+            const double t = std::ceil((double)nn / s.clusters) * s.time;
+            const double alone = nn <= s.clusters / s.per_sm ? s.time / s.per_sm : t;
+            const double v = std::min(t, std::max(alone, 0.0));
+            if (shapes[0].csz == 0 || v < 0.98 * best) {
+                best = v;
+                shapes[0] = s;
+            }
+        }
+        return true;
+    }
+    double total = 0.0;
+    auto sm_time = [&](int k, const KryShape& s) {
+        return (double)(first[k + 1] - first[k]) * s.time * dims[k].dims[2] / s.clusters;
+    };
+    for (int k = 0; k < nc; ++k) {
+        for (const KryShape& s : cand[k])
+            if (shapes[k].csz == 0 || sm_time(k, s) < 0.98 * sm_time(k, shapes[k])) shapes[k] = s;
+        total += sm_time(k, shapes[k]);
+    }
+    for (int k = 0; k < nc; ++k)
+        for (const KryShape& s : cand[k])
+            if (shapes[k].time * dims[k].dims[2] > 0.7 * total && s.time < 0.9 * shapes[k].time && s.csz > shapes[k].csz) {
+                total += sm_time(k, s) - sm_time(k, shapes[k]);
+                shapes[k] = s;
+            }
+    return true;
+}
+
+// Launch parameters of every class (scratch and list pointers are set by
+// the caller) and the scratch they need side by side.
+size_t kry_params(const Ham& H, const std::vector<int>& first, const std::vector<KryShape>& shapes,
+                  const std::vector<NodeDesc>& dims, std::vector<KryClass>& out) {
+    const bool nl = H.nonlocal && H.n_atoms > 0;
+    const double scale = kry_scale(H);
+    size_t total = 0;
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    out.clear();
+    for (size_t k = 0; k < shapes.size(); ++k) {
+        KryClass c;
+        std::memset(&c.P, 0, sizeof(c.P));
+        const KryShape& s = shapes[k];
+        KrylovParams& P = c.P;
+        const size_t items = (size_t)s.depth * ((dims[k].dims[0] + 1) / 2) * dims[k].dims[1];   // pairs of points
+        c.csz = s.csz;
+        c.block = s.block;
+        c.smem = s.smem;
+        P.n_work = first[k + 1] - first[k];
+        c.grid = std::min(P.n_work, s.clusters) * s.csz;
+        for (int d = 0; d < 3; ++d) {
+            P.n[d] = H.n[d];
+            P.periodic[d] = H.periodic[d];
+        }
+        P.V = H.V;
+        kry_operator(P, H, scale);
+        P.n_atoms = H.n_atoms;
+        P.proj_i0 = H.proj_i0;
+        P.proj_len = H.proj_len;
+        P.proj_rows = H.proj_rows;
+        P.proj_fx = H.proj_fx;
+        P.proj_fxc = H.proj_fxc;
+        P.rec_words = nl ? std::max(1, H.pl_max) : 0;   // two entries a word; a pair meets up to 2 pl_max rows
+        P.smem_bytes = (int)s.smem;
+        const int win_y = std::min(2 * (int)std::floor(H.proj_rc / H.h[1]) + 2, kMaxProjWin);
+        const size_t local = (size_t)std::min<long long>(H.n_atoms, kMaxLocalProjAtoms);
+        P.row_cap = nl ? (int)std::min<size_t>(2 * items * H.pl_max, local * win_y * s.depth * 2) : 0;
+        P.off_up = up(items * sizeof(int4));
+        P.off_w = P.off_up + up(items * sizeof(int4));
+        P.off_rec = P.off_w + up(items * sizeof(longlong2));
+        P.win_x = nl ? std::min(2 * (int)std::floor(H.proj_rc / H.h[0]) + 2, kMaxProjWin) : 0;
+        P.off_rows = P.off_rec + up(items * P.rec_words * sizeof(uint4));
+        P.off_ktab = P.off_rows + up((size_t)P.row_cap * 32);
+        P.off_xtab = P.off_ktab + up(((size_t)P.row_cap + 1) * 16);
+        P.off_chunk = P.off_xtab + up((local * P.win_x + 1) * 16);
+        P.off_cpart = P.off_chunk + up(((size_t)P.row_cap / kKryChunkRows + local + 1) * 16);
+        P.cta_bytes = P.off_cpart + up(nl ? kMaxLocalProjAtoms * 4 * 32 : 0);
+        for (int d = 0; d < 3; ++d)
+            for (int o = 0; o < kKryMaxQ; ++o) P.coef[d][o] = H.coef[d][o];
+        P.dV = H.dV;
+        P.e_s = H.e_s;
+        P.e_p = H.e_p;
+        P.pl_ptr = H.pl_ptr;
+        P.pl_atom = H.pl_atom;
+        P.pl_val64 = H.pl_val64;
+        total += P.cta_bytes * c.grid;
+        out.push_back(c);
+    }
+    return total;
+}
+
+void kry_scratch(std::vector<KryClass>& cls, char* base, const int* list, unsigned int* counters,
+                 const NodeDesc* nodes, const std::vector<int>& first) {
+    for (size_t k = 0; k < cls.size(); ++k) {
+        KrylovParams& P = cls[k].P;
+        P.scratch = base;
+        base += P.cta_bytes * cls[k].grid;
+        P.list = list + first[k];
+        P.nodes = nodes;
+        P.work_counter = counters + k;
+    }
+}
+
+cudaError_t kry_side_create(KrySide& d) {
+    if (d.fork) return cudaSuccess;
+    for (int i = 0; i < kKryStreams - 1; ++i) {
+        cudaError_t e = cudaStreamCreateWithFlags(&d.s[i], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&d.join[i], cudaEventDisableTiming);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaEventCreateWithFlags(&d.fork, cudaEventDisableTiming);
+}
+
+void kry_side_free(KrySide& d) {
+    for (int i = 0; i < kKryStreams - 1; ++i) {
+        if (d.s[i]) cudaStreamDestroy(d.s[i]);
+        if (d.join[i]) cudaEventDestroy(d.join[i]);
+    }
+    if (d.fork) cudaEventDestroy(d.fork);
+    d = KrySide();
+}
+
+// All classes at once: the first on `stream`, the others on side streams
+// forked from and joined to it (classes of small regions fill the SMs the
+// large ones leave).
+cudaError_t kry_launch(const std::vector<KryClass>& cls, const Ham& H, KrySide& side, cudaStream_t stream) {
+    const int nl = H.nonlocal && H.n_atoms > 0 ? 1 : 0;
+    const int ns = std::min<int>(kKryStreams, (int)cls.size());
+    cudaError_t e = cudaSuccess;
+    if (ns > 1) {
+        e = kry_side_create(side);
+        if (e == cudaSuccess) e = cudaEventRecord(side.fork, stream);
+        for (int i = 1; i < ns && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(side.s[i - 1], side.fork, 0);
+    }
+    for (size_t k = 0; k < cls.size() && e == cudaSuccess; ++k) {
+        const int i = (int)(k % ns);
+        e = launch_krylov(cls[k].P, H.q, nl, cls[k].csz, cls[k].grid, cls[k].block, cls[k].smem,
+                          i == 0 ? stream : side.s[i - 1]);
+    }
+    for (int i = 1; i < ns && e == cudaSuccess; ++i) {
+        e = cudaEventRecord(side.join[i - 1], side.s[i - 1]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, side.join[i - 1], 0);
+    }
+    return e;
+}
+
+}  // namespace
+}  // namespace md
+
 // ---------------------------------------------------------------------------
 // Plans: one prepared batched solve, replayed as a CUDA graph.
 // ---------------------------------------------------------------------------
@@ -277,6 +590,8 @@ struct md_plan {
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     bool launched = false;
+    std::vector<md::KryClass> kry;     // node-shared Krylov solve: one launch per size class
+    md::KrySide side;
 };
 
 namespace md {
@@ -306,6 +621,7 @@ void plan_free(md_plan* pl) {
             else cudaFree(p);
         }
     if (pl->own_scratch && pl->scratch) cudaFree(pl->scratch);
+    kry_side_free(pl->side);
     delete pl;
 }
 
@@ -573,6 +889,33 @@ struct FusedArgs {
     const long long* dm_off;
 };
 
+// Reset the work counters, solve, accumulate rho and e.
+cudaError_t plan_enqueue(md_plan* pl, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(pl->d_counter, 0, kKryClasses * sizeof(unsigned int), s);
+    if (e != cudaSuccess) return e;
+    if (!pl->kry.empty()) e = kry_launch(pl->kry, *pl->H, pl->side, s);
+    else e = launch_shape(pl, pl->P, Shape{pl->variant, pl->block, pl->per_sm, pl->cluster}, pl->grid, s);
+    if (e != cudaSuccess) return e;
+    return launch_accumulate((int)pl->nn, pl->Pn, pl->d_xsrc, pl->d_z, pl->d_w, pl->H->dV, pl->rho_out, pl->e_out, s);
+}
+
+cudaError_t plan_capture(md_plan* pl) {
+    if (pl->exec) cudaGraphExecDestroy(pl->exec);
+    if (pl->graph) cudaGraphDestroy(pl->graph);
+    pl->exec = nullptr;
+    pl->graph = nullptr;
+    if (pl->kry.size() > 1) {   // made outside the capture
+        const cudaError_t e = kry_side_create(pl->side);
+        if (e != cudaSuccess) return e;
+    }
+    cudaError_t e = cudaStreamBeginCapture(pl->cap, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    const cudaError_t e1 = plan_enqueue(pl, pl->cap);
+    const cudaError_t e2 = cudaStreamEndCapture(pl->cap, &pl->graph);
+    if (e1 != cudaSuccess || e2 != cudaSuccess) return e1 != cudaSuccess ? e1 : e2;
+    return cudaGraphInstantiate(&pl->exec, pl->graph, 0);
+}
+
 // direct: launch at once on `stream` without a graph and without
 // synchronising it (device temporaries allocated and freed stream-ordered,
 // uploads staged through the handle's pinned buffers); the caller frees the
@@ -659,6 +1002,17 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
         return ca > cb;
     });
     const long long n_work = (long long)sys.size();
+    // one Krylov sequence per node for all its poles (md_krylov.cu) unless
+    // the caller asks for a kernel or launch shape, or needs the solution
+    // vectors, or a region does not fit
+    std::vector<int> korder, kfirst;
+    std::vector<KryShape> kshape;
+    std::vector<NodeDesc> kdims;
+    // (FP64 solves keep the per-pole kernel: with and without a checkpoint they
+    // return the same bits)
+    const bool kry = opts.kernel == 0 && opts.block == 0 && opts.ctas_per_sm == 0 && !ckpt && !fused &&
+                     (opts.precision == MD_PREC_MIXED || ms) && Pn <= kKryMaxPoles && kry_scale(H) > 0.0 && kry_classes(H, R, korder, kfirst, kshape, kdims);
+    const size_t kneed = kry ? kry_params(H, kfirst, kshape, kdims, pl->kry) : 0;
     auto dmalloc = [&](auto** p, size_t b) {
         return direct ? cudaMallocAsync((void**)p, b, stream) : cudaMalloc((void**)p, b);
     };
@@ -671,7 +1025,11 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     PTRY(dmalloc(&pl->d_xsrc, n_sys * sizeof(double2)));
     PTRY(dmalloc(&pl->d_z, Pn * sizeof(double2)));
     PTRY(dmalloc(&pl->d_w, Pn * sizeof(double2)));
-    PTRY(dmalloc(&pl->d_counter, sizeof(unsigned int)));
+    PTRY(dmalloc(&pl->d_counter, kKryClasses * sizeof(unsigned int)));
+    if (kry) {   // the work list of the classes takes the place of the system list
+        static_assert(sizeof(SysDesc) >= sizeof(int), "node list fits the system list");
+        std::memcpy(sys.data(), korder.data(), nn * sizeof(int));
+    }
     std::vector<long long> ckoff;
     if (ckpt) {
         ckoff.resize(n_sys);
@@ -757,14 +1115,14 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     P.n_rel = pl->d_nrel;
 
     const int max_plane = R.max_dim[0] * R.max_dim[1];
-    const bool zm_ok = zm_supported(opts.precision, H.q) && !R.any_ring && !ms && !fused;
+    const bool zm_ok = !kry && zm_supported(opts.precision, H.q) && !R.any_ring && !ms && !fused;
     P.zm_m0 = R.max_dim[0];
     P.zm_m1 = R.max_dim[1];
     if (zm_ok) pl->smem = zm_smem_bytes(H.q, R.max_dim[0], R.max_dim[1]);
     // the cluster kernel: mixed precision, no whole-axis rings, per-pole COCG
     // (regions with at most 255 points along y: the row records hold the row in 8 bits)
     P.cl_wx = P.nonlocal ? std::min(2 * (int)std::floor(H.proj_rc / H.h[0]) + 2, kMaxProjWin) : 0;
-    const bool cl_ok = cl_supported(opts.precision, H.q) && !R.any_ring && !ms && R.max_dim[1] <= 255 &&
+    const bool cl_ok = !kry && cl_supported(opts.precision, H.q) && !R.any_ring && !ms && R.max_dim[1] <= 255 &&
                        cl_geometry(H.q, R.max_dim[2], max_plane, dev,
                                    opts.kernel == 3 && opts.ctas_per_sm > 0 ? std::min(opts.ctas_per_sm, 8) : 0,
                                    P.cl_wx, pl->cluster, P.cl_slab, pl->cl_smem, pl->cl_block, P.cl_xcap);
@@ -779,7 +1137,7 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     }
     // scratch sized for the widest candidate (3 CTAs per SM, or one slot per SM for clusters)
     const int max_ctas = (int)std::min<long long>((long long)n_sm * 3, n_work);
-    const size_t need = std::max(P.slot_bytes * (size_t)max_ctas,
+    const size_t need = kry ? kneed : std::max(P.slot_bytes * (size_t)max_ctas,
                                  cl_ok ? cl_slot_bytes(P.n_max, pl->cluster, P.cl_slab, P.nonlocal, P.cl_row_cap, P.cl_key_cap) *
                                              (size_t)std::min<long long>(n_sm, n_work)
                                        : 0);
@@ -801,6 +1159,25 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
         PTRY(cudaMalloc(&pl->scratch, need));
     }
     P.scratch = (char*)pl->scratch;
+    if (kry) {
+        for (KryClass& c : pl->kry) {
+            KrylovParams& K = c.P;
+            K.timeout_ns = P.timeout_ns;
+            K.P = Pn;
+            K.z = pl->d_z;
+            K.tol = opts.tol;
+            K.maxit = opts.maxit;
+            K.x_src = pl->d_xsrc;
+            K.status = pl->d_status;
+            K.iters = pl->d_iters;
+            K.resid = pl->d_resid;
+            K.n_rel = pl->d_nrel;
+            K.check = opts.precision == MD_PREC_MIXED;
+        }
+        kry_scratch(pl->kry, (char*)pl->scratch, (const int*)pl->d_sys, pl->d_counter, pl->d_nodes, kfirst);
+        pl->block = pl->kry[0].block;
+        pl->grid = pl->kry[0].grid;
+    }
 
     Shape shape{0, opts.block > 0 ? opts.block : 512, opts.ctas_per_sm > 0 ? opts.ctas_per_sm : 0};
     if (opts.kernel == 3) {   // the cluster kernel, forced
@@ -823,7 +1200,7 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
         shape.variant = K;
         if (shape.per_sm <= 0) shape.per_sm = 1;
     }
-    if (opts.block <= 0 && opts.kernel != 3) {
+    if (!kry && opts.block <= 0 && opts.kernel != 3) {
         const std::vector<Shape> cands = candidate_shapes(pl, zm_ok, max_plane);
         md_status ts = autotune(pl, n_sm, cands, need, shape, stream);
         if (ts != MD_OK) return fail(ts);
@@ -832,35 +1209,24 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
         if (shape.per_sm <= 0) shape.per_sm = std::max(1, 1024 / shape.block);
         shape.per_sm = std::min(shape.per_sm, opts.precision == MD_PREC_MIXED && shape.variant == 0 ? 3 : 2);
     }
-    pl->variant = shape.variant;
-    pl->block = shape.block;
-    pl->per_sm = shape.per_sm;
-    pl->cluster = shape.cluster;
-    pl->grid = grid_of(shape, n_sm, n_work);
+    if (!kry) {
+        pl->variant = shape.variant;
+        pl->block = shape.block;
+        pl->per_sm = shape.per_sm;
+        pl->cluster = shape.cluster;
+        pl->grid = grid_of(shape, n_sm, n_work);
+    }
 
-    if (direct) {   // [reset counter, solver, accumulation] on the caller's stream, now
-        PTRY(cudaMemsetAsync(pl->d_counter, 0, sizeof(unsigned int), stream));
-        PTRY(launch_shape(pl, P, Shape{pl->variant, pl->block, pl->per_sm, pl->cluster}, pl->grid, stream));
-        PTRY(launch_accumulate((int)nn, Pn, pl->d_xsrc, pl->d_z, pl->d_w, H.dV, rho_out, e_out, stream));
+    if (direct) {   // [reset counters, solver, accumulation] on the caller's stream, now
+        PTRY(plan_enqueue(pl, stream));
         if (!H.scratch_ev) PTRY(cudaEventCreateWithFlags(&H.scratch_ev, cudaEventDisableTiming));
         PTRY(cudaEventRecord(H.scratch_ev, stream));
         pl->launched = true;
         *out = pl;
         return MD_OK;
     }
-    // capture [reset counter, solver, accumulation] once; launches replay it
-    PTRY(cudaStreamBeginCapture(pl->cap, cudaStreamCaptureModeThreadLocal));
-    {
-        cudaError_t e1 = cudaMemsetAsync(pl->d_counter, 0, sizeof(unsigned int), pl->cap);
-        cudaError_t e2 = launch_shape(pl, P, Shape{pl->variant, pl->block, pl->per_sm, pl->cluster}, pl->grid, pl->cap);
-        cudaError_t e3 = launch_accumulate((int)nn, Pn, pl->d_xsrc, pl->d_z, pl->d_w, H.dV, rho_out, e_out, pl->cap);
-        cudaError_t e4 = cudaStreamEndCapture(pl->cap, &pl->graph);
-        PTRY(e1);
-        PTRY(e2);
-        PTRY(e3);
-        PTRY(e4);
-    }
-    PTRY(cudaGraphInstantiate(&pl->exec, pl->graph, 0));
+    // capture the same once; launches replay it
+    PTRY(plan_capture(pl));
 #undef PTRY
     *out = pl;
     return MD_OK;
@@ -869,6 +1235,15 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
 md_status plan_launch(md_plan* pl, cudaStream_t stream) {
     if (!pl) return set_error(MD_ERR_INVALID, "plan is NULL");
     if (pl->n_sys == 0) return MD_OK;
+    if (!pl->kry.empty()) {
+        // md_hamiltonian_set_potential may have moved the spectral bounds
+        // that fix the scale of the fixed-point operator
+        const double scale = kry_scale(*pl->H);
+        if (scale > 0.0 && scale != pl->kry[0].P.scale) {
+            for (KryClass& c : pl->kry) kry_operator(c.P, *pl->H, scale);
+            PLAN_TRY(plan_capture(pl));
+        }
+    }
     PLAN_TRY(cudaEventRecord(pl->ev0, stream));
     PLAN_TRY(cudaGraphLaunch(pl->exec, stream));
     PLAN_TRY(cudaEventRecord(pl->ev1, stream));
@@ -1475,7 +1850,14 @@ extern "C" md_status md_lssgq_rules(const md_hamiltonian* ham, const md_nodes* n
     // every call but an asynchronous md_density ends synchronised with its
     // stream; wait for the last of those before using the scratch
     LTRY(scratch_idle(H));
-    const size_t need = P.slot_bytes * (size_t)grid;
+    // the fixed-point kernel (md_krylov.cu) unless the caller gives a CTA size
+    // or a region does not fit
+    std::vector<int> korder, kfirst;
+    std::vector<KryShape> kshape;
+    std::vector<NodeDesc> kdims;
+    std::vector<KryClass> kcls;
+    const bool kry = opts->block == 0 && kry_scale(H) > 0.0 && kry_classes(H, R, korder, kfirst, kshape, kdims);
+    const size_t need = kry ? kry_params(H, kfirst, kshape, kdims, kcls) : P.slot_bytes * (size_t)grid;
     if (need > H.scratch_bytes) {
         LTRY(cudaStreamSynchronize(s));
         if (H.scratch) cudaFree(H.scratch);
@@ -1509,9 +1891,10 @@ extern "C" md_status md_lssgq_rules(const md_hamiltonian* ham, const md_nodes* n
     int* d_kused = (int*)(lz + o_kused);
     int* d_status = (int*)(lz + o_status);
     unsigned int* d_counter = (unsigned int*)(lz + o_counter);
+    if (kry) std::memcpy(sys.data(), korder.data(), nn * sizeof(int));
     LTRY(cudaMemcpyAsync(d_sys, sys.data(), nn * sizeof(SysDesc), cudaMemcpyHostToDevice, s));
     LTRY(cudaMemcpyAsync(d_nodes, R.desc.data(), nn * sizeof(NodeDesc), cudaMemcpyHostToDevice, s));
-    LTRY(cudaMemsetAsync(d_counter, 0, sizeof(unsigned int), s));
+    LTRY(cudaMemsetAsync(d_counter, 0, kKryClasses * sizeof(unsigned int), s));
     LTRY(cudaMemsetAsync(d_kused, 0, nn * sizeof(int), s));
     P.sys = d_sys;
     P.nodes = d_nodes;
@@ -1523,7 +1906,25 @@ extern "C" md_status md_lssgq_rules(const md_hamiltonian* ham, const md_nodes* n
     L.beta = d_beta;
     L.k_used = d_kused;
     L.status = d_status;
-    LTRY(launch_lanczos(P, L, opts->precision, grid, block, s));
+    KrySide side;
+    if (kry) {
+        for (KryClass& c : kcls) {
+            KrylovParams& Q = c.P;
+            Q.timeout_ns = P.timeout_ns;
+            Q.K = K;
+            Q.breakdown_tol = L.breakdown_tol;
+            Q.alpha = L.alpha;
+            Q.beta = L.beta;
+            Q.k_used = L.k_used;
+            Q.node_status = L.status;
+        }
+        kry_scratch(kcls, (char*)H.scratch, (const int*)d_sys, d_counter, d_nodes, kfirst);
+        const cudaError_t e = kry_launch(kcls, H, side, s);
+        kry_side_free(side);
+        LTRY(e);
+    } else {
+        LTRY(launch_lanczos(P, L, opts->precision, grid, block, s));
+    }
     LTRY(launch_gauss_rules((int)nn, L, lambda_out, weight_out, s));
     if (k_used_out)
         LTRY(cudaMemcpyAsync(k_used_out, d_kused, nn * sizeof(int), cudaMemcpyDeviceToDevice, s));

@@ -23,6 +23,7 @@
 
 #include "md_device.cuh"
 #include "md_internal.h"
+#include "md_krylov.h"
 
 namespace md {
 
@@ -554,6 +555,12 @@ md_status build_hamiltonian_device(Ham& H, const md_atoms* atoms, const md_pot_p
                                                             H.dV, H.proj_C, H.proj_C32, H.proj_absum);
             MD_CUDA_TRY(cudaGetLastError());
         }
+        MD_CUDA_TRY(cudaMalloc(&H.proj_fx, tab * sizeof(int4)));
+        MD_CUDA_TRY(cudaMalloc(&H.proj_fxc, 4 * na * sizeof(double)));
+        MD_CUDA_TRY(cudaMalloc(&d_overflow, 2 * sizeof(int)));
+        MD_CUDA_TRY(cudaMemsetAsync(d_overflow, 0, 2 * sizeof(int), stream));
+        MD_CUDA_TRY(launch_proj_fixed(na, H.proj_len, H.proj_d, H.proj_g, H.proj_C, H.dV, H.e_s, H.e_p, H.proj_fx,
+                                      H.proj_fxc, d_overflow + 1, stream));
         // per-point lists: count, host scan, fill
         build_cells(H, xyz, H.proj_rc, cstart_p, cids_p, ncp, cellp);
         MD_CUDA_TRY(cudaFree(d_cstart));
@@ -567,25 +574,25 @@ md_status build_hamiltonian_device(Ham& H, const md_atoms* atoms, const md_pot_p
         }
         ca.start = d_cstart;
         MD_CUDA_TRY(cudaMalloc(&d_count, (N + 1) * sizeof(int)));
-        MD_CUDA_TRY(cudaMalloc(&d_overflow, sizeof(int)));
-        MD_CUDA_TRY(cudaMemsetAsync(d_overflow, 0, sizeof(int), stream));
         k_proj_lists<false><<<blocks, threads, 0, stream>>>(g, ca, H.proj_i0, H.proj_len, H.proj_rows,
                                                             H.proj_d, H.proj_g, H.proj_C, N, d_count,
                                                             nullptr, nullptr, nullptr, d_overflow);
         MD_CUDA_TRY(cudaGetLastError());
         {
             std::vector<int> cnt(N + 1, 0);
-            int ovf = 0;
+            int ovf[2] = {0, 0};
             MD_CUDA_TRY(cudaMemcpyAsync(cnt.data(), d_count, N * sizeof(int), cudaMemcpyDeviceToHost, stream));
-            MD_CUDA_TRY(cudaMemcpyAsync(&ovf, d_overflow, sizeof(int), cudaMemcpyDeviceToHost, stream));
+            MD_CUDA_TRY(cudaMemcpyAsync(ovf, d_overflow, sizeof(ovf), cudaMemcpyDeviceToHost, stream));
             MD_CUDA_TRY(cudaStreamSynchronize(stream));
-            if (ovf) {
+            H.proj_fx_ok = ovf[1] == 0;
+            if (ovf[0]) {
                 st = set_error(MD_ERR_INVALID, "md_build_hamiltonian: more than 16 projector atoms at one grid point");
                 goto fail;
             }
             long long run = 0;
             for (long long i = 0; i < N; ++i) {
                 const long long c = cnt[i];
+                H.pl_max = std::max(H.pl_max, cnt[i]);
                 if (run > 2147483647LL - 16) {
                     st = set_error(MD_ERR_INVALID, "md_build_hamiltonian: too many projector entries (2^31)");
                     goto fail;

@@ -68,6 +68,10 @@ struct Ham {
     float4* pl_val32 = nullptr;       // [nnz] (p_s, p_x, p_y, p_z) at the point, FP32
     double2* pl_val64 = nullptr;      // [nnz][2] the same in FP64
     long long pl_nnz = 0;
+    int pl_max = 0;                   // largest list length of a point
+    int4* proj_fx = nullptr;          // [n_atoms][3][kMaxProjWin] unit tables in fixed point (md_krylov.h)
+    double* proj_fxc = nullptr;       // [n_atoms][4] their coefficients
+    bool proj_fx_ok = false;          // every atom's normalisation is in range
 
     bool bounds_valid = false;
     double emin = 0.0, emax = 0.0;
