@@ -433,7 +433,8 @@ bool kry_classes(const Ham& H, const Regions& R, std::vector<int>& order, std::v
 // Launch parameters of every class (scratch and list pointers are set by
 // the caller) and the scratch they need side by side.
 size_t kry_params(const Ham& H, const std::vector<int>& first, const std::vector<KryShape>& shapes,
-                  const std::vector<NodeDesc>& dims, std::vector<KryClass>& out) {
+                  const std::vector<NodeDesc>& dims, std::vector<KryClass>& out, int vec_poles = 0,
+                  bool own_x = false) {
     const bool nl = H.nonlocal && H.n_atoms > 0;
     const double scale = kry_scale(H);
     size_t total = 0;
@@ -468,7 +469,8 @@ size_t kry_params(const Ham& H, const std::vector<int>& first, const std::vector
         const size_t local = (size_t)std::min<long long>(H.n_atoms, kMaxLocalProjAtoms);
         P.row_cap = nl ? (int)std::min<size_t>(2 * items * H.pl_max, local * win_y * s.depth * 2) : 0;
         P.off_up = up(items * sizeof(int4));
-        P.off_w = P.off_up + up(items * sizeof(int4));
+        P.vec = vec_poles > 0;
+        P.off_w = P.off_up + up(items * sizeof(int4) * (P.vec ? kKryVec : 1));
         P.off_rec = P.off_w + up(items * sizeof(longlong2));
         P.win_x = nl ? std::min(2 * (int)std::floor(H.proj_rc / H.h[0]) + 2, kMaxProjWin) : 0;
         P.off_rows = P.off_rec + up(items * P.rec_words * sizeof(uint4));
@@ -476,7 +478,11 @@ size_t kry_params(const Ham& H, const std::vector<int>& first, const std::vector
         P.off_xtab = P.off_ktab + up(((size_t)P.row_cap + 1) * 16);
         P.off_chunk = P.off_xtab + up((local * P.win_x + 1) * 16);
         P.off_cpart = P.off_chunk + up(((size_t)P.row_cap / kKryChunkRows + local + 1) * 16);
-        P.cta_bytes = P.off_cpart + up(nl ? kMaxLocalProjAtoms * 4 * 32 : 0);
+        P.off_x = P.off_cpart + up(nl ? kMaxLocalProjAtoms * 4 * 32 : 0);
+        P.off_p = P.off_x + up(own_x ? items * vec_poles * 2 * sizeof(double2) : 0);
+        P.off_hist = P.off_p + up(items * vec_poles * 2 * sizeof(double2));
+        P.off_coef = P.off_hist + (P.vec ? (size_t)kKryVec * kKryMaxPoles * 32 : 0);
+        P.cta_bytes = P.off_hist + up(P.vec ? kry_vec_bytes(vec_poles) : 0);
         for (int d = 0; d < 3; ++d)
             for (int o = 0; o < kKryMaxQ; ++o) P.coef[d][o] = H.coef[d][o];
         P.dV = H.dV;
@@ -1003,16 +1009,16 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     });
     const long long n_work = (long long)sys.size();
     // one Krylov sequence per node for all its poles (md_krylov.cu) unless
-    // the caller asks for a kernel or launch shape, or needs the solution
-    // vectors, or a region does not fit
+    // the caller asks for a kernel or launch shape or a region does not fit
     std::vector<int> korder, kfirst;
     std::vector<KryShape> kshape;
     std::vector<NodeDesc> kdims;
-    // (FP64 solves keep the per-pole kernel: with and without a checkpoint they
-    // return the same bits)
-    const bool kry = opts.kernel == 0 && opts.block == 0 && opts.ctas_per_sm == 0 && !ckpt && !fused &&
-                     (opts.precision == MD_PREC_MIXED || ms) && Pn <= kKryMaxPoles && kry_scale(H) > 0.0 && kry_classes(H, R, korder, kfirst, kshape, kdims);
-    const size_t kneed = kry ? kry_params(H, kfirst, kshape, kdims, pl->kry) : 0;
+    // (mixed shifted COCG keeps its FP32 kernel: it needs no more than FP32 moves a step)
+    const bool kry = opts.kernel == 0 && opts.block == 0 && opts.ctas_per_sm == 0 && Pn <= kKryMaxPoles &&
+                     !(ms && opts.precision == MD_PREC_MIXED) &&
+                     kry_scale(H) > 0.0 && kry_classes(H, R, korder, kfirst, kshape, kdims);
+    const bool kvec = ckpt || fused;   // the solution vectors are needed
+    const size_t kneed = kry ? kry_params(H, kfirst, kshape, kdims, pl->kry, kvec ? Pn : 0, !ckpt) : 0;
     auto dmalloc = [&](auto** p, size_t b) {
         return direct ? cudaMallocAsync((void**)p, b, stream) : cudaMalloc((void**)p, b);
     };
@@ -1173,6 +1179,14 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
             K.resid = pl->d_resid;
             K.n_rel = pl->d_nrel;
             K.check = opts.precision == MD_PREC_MIXED;
+            K.ckpt = P.ckpt;
+            K.ckpt_off = P.ckpt_sys_off;
+            K.fused_dLdV = P.fused_dLdV;
+            K.fused_a = P.fused_a;
+            K.fused_b = P.fused_b;
+            K.w = P.w;
+            K.dm_rows = P.dm_rows;
+            K.dm_off = P.dm_off;
         }
         kry_scratch(pl->kry, (char*)pl->scratch, (const int*)pl->d_sys, pl->d_counter, pl->d_nodes, kfirst);
         pl->block = pl->kry[0].block;
@@ -1856,7 +1870,8 @@ extern "C" md_status md_lssgq_rules(const md_hamiltonian* ham, const md_nodes* n
     std::vector<KryShape> kshape;
     std::vector<NodeDesc> kdims;
     std::vector<KryClass> kcls;
-    const bool kry = opts->block == 0 && kry_scale(H) > 0.0 && kry_classes(H, R, korder, kfirst, kshape, kdims);
+    // (FP32 vectors keep their own kernel: at 24 B a point-step it is faster)
+    const bool kry = opts->precision == MD_PREC_FP64 && opts->block == 0 && kry_scale(H) > 0.0 && kry_classes(H, R, korder, kfirst, kshape, kdims);
     const size_t need = kry ? kry_params(H, kfirst, kshape, kdims, kcls) : P.slot_bytes * (size_t)grid;
     if (need > H.scratch_bytes) {
         LTRY(cudaStreamSynchronize(s));

@@ -46,6 +46,7 @@
 #include <cuda_runtime.h>
 
 #include <cfloat>
+#include <cstddef>
 #include <cstdint>
 
 #include "md_krylov.h"
@@ -167,8 +168,18 @@ struct KShared {
     double s0, inv0;              // ||u||^2, 1/||u||^2
     double a_hat, b2_hat;         // alpha, beta^2 of the step just taken (in units of scale)
     double scale0;                // Lanczos breakdown scale
-    int e_prev;
+    int e_hat;                    // its e
     int nonfinite;
+};
+struct VecHead {      // one pole's update of its solution vector
+    double sw, sv;    // powers of two the coefficients were divided by
+    double2 om, nu;
+    int act, first;
+};
+struct KSharedVec {
+    int4 co[4 * kKryVec];         // coefficients of the pole in hand
+    VecHead head;
+    double2 cp[kKryMaxPoles];     // pole factors of the outputs
 };
 struct KSharedNl {
     int n_local, n_rows, n_chunks, n_tab, over;
@@ -423,7 +434,6 @@ __device__ __forceinline__ int4 row_factors(const KRow* row, const int2* cl) {
 struct SlabArgs {
     const int2* U;
     int4* Vp;            // [depth][npc] V limbs of the pair
-    int4* Up;            // u_prev limbs
     longlong2* Wp;       // w
     const uint4* Rec;    // [depth][npc][rec_words]
     int m0, m1, npx, npc, n_items, pitch, pp;
@@ -485,8 +495,8 @@ __device__ __forceinline__ void stencil(const KrylovParams& P, const SlabArgs& A
 // and 19 warps at 96 registers are the faster trade.
 template <int Q, bool kNl>
 __device__ __forceinline__ void slab_apply(const KrylovParams& P, const SlabArgs& A, const int4* ktab,
-                                           const int4* xtab, int nw, int2 g, long long& hh1, long long& l1,
-                                           long long& hh2, long long& l2) {
+                                           const int4* xtab, const int4* u_prev, int nw, int2 g, long long& hh1,
+                                           long long& l1, long long& hh2, long long& l2) {
     long long x1 = 0, y1 = 0, x2 = 0;
     float q1 = 0.f, q2 = 0.f;
     int steps = 0;
@@ -495,7 +505,7 @@ __device__ __forceinline__ void slab_apply(const KrylovParams& P, const SlabArgs
         const int i = i0 + (int)(threadIdx.x & 31);
         const bool act = i < A.n_items;
         const int item = act ? i : A.n_items - 1;
-        const int4 v = A.Vp[item], um = A.Up[item];   // from L2, used after the stencil sums
+        const int4 v = A.Vp[item], um = u_prev[item];   // from L2, used after the stencil sums
         uint4 rc = make_uint4(0u, 0u, 0u, 0u);
         if (kNl) rc = A.Rec[(size_t)item * P.rec_words];
         const int d = (int)fdiv((uint32_t)item, A.div_pc), pc = item - d * A.npc;
@@ -544,7 +554,8 @@ __device__ __forceinline__ double limbs(int hi, int lo) { return fma((double)hi,
 // xsum exchanges them over the cluster.
 template <int Q, bool kNl, class F>
 __device__ __noinline__ double check_step(const KrylovParams& P, const SlabArgs& A, const int lo[3], int z0,
-                                          const KSharedNl& S, double* c, int2 g2, F&& xsum) {
+                                          const KSharedNl& S, double* c, const int4* u_prev, int2 g2,
+                                          F&& xsum) {
     const double g = limbs(g2.x, g2.y);
     auto global_point = [&](int item, int& d, int& b, int& a) {
         d = item / A.npc;
@@ -612,7 +623,7 @@ __device__ __noinline__ double check_step(const KrylovParams& P, const SlabArgs&
                     y += P.dV * (P.e_s * v.x * c[4 * s] + P.e_p * (v.y * c[4 * s + 1] + q.x * c[4 * s + 2] + q.y * c[4 * s + 3]));
                 }
             }
-            const int4 um = A.Up[item];
+            const int4 um = u_prev[item];
             const longlong2 w = A.Wp[item];
             const double t = y * inv - g * (i ? limbs(um.z, um.w) : limbs(um.x, um.y)) - (double)(i ? w.y : w.x) * 0x1p-62;
             s2 += t * t;
@@ -629,26 +640,143 @@ struct PoleState {
     double fr, fi;     // zeta^2
     double gr, gi;     // x(j) * scale
     double rn;         // ||r||
-    int conv;
+    int conv;          // step at which ||r|| <= tol
+    int frz;           // step at which the solution vector is complete (||r|| <= kFreeze tol)
+    double cr, ci;     // chi = zeta / ||u||
+    double mr, mi;     // m of the last step of the chunk before
 };
+// Solution vectors are carried on until ||r|| <= 0.3 tol: the other poles of
+// the node go on anyway, and the slowest pays a few steps.
+constexpr double kFreeze = 0.3;
 
-__device__ __forceinline__ void pole_step(PoleState& s, double a, double b2) {
+__device__ __forceinline__ void pole_step(PoleState& s, double a, double b2, bool sum) {
     const double dr = a - s.zr - s.er, di = -s.zi - s.ei;
     const double inv = 1.0 / (dr * dr + di * di);
     const double ir = dr * inv, ii = -di * inv;
     const double qr = s.fr * ir - s.fi * ii, qi = s.fr * ii + s.fi * ir;
-    s.gr += qr;
-    s.gi += qi;
+    if (sum) {
+        s.gr += qr;
+        s.gi += qi;
+    }
     s.er = b2 * ir;
     s.ei = b2 * ii;
     s.fr = qr * s.er - qi * s.ei;
     s.fi = qr * s.ei + qi * s.er;
 }
 
+// Solution vectors.  In terms of the vectors u_k as kept, COCG's directions
+// and iterates of a pole are
+//   p_k = u_k - m_{k-1} p_{k-1},   m_k = 2^{e_k} beta_k^2 / d_k,
+//   x  += c_k p_k,                 c_k = chi_k / d_k,  chi_{k+1} = -2^{-e_k} c_k.
+// kKryVec steps are applied at a time: with u_{s+1} .. u_e kept,
+//   x <- x + sum_j w_j u_j + omega p_s,   w_j = c_j - m_j w_{j+1}, omega = -m_s w_{s+1},
+//   p <-     sum_j v_j u_j + nu p_s,      v_j = -m_j v_{j+1},      nu = -m_s v_{s+1}.
+struct VecHist {
+    double2 c, m;
+};
+
+// Coefficients of a pole's update as fixed point: {hi, (float)hi, (float)lo}
+// of Re w, Im w, Re v, Im v for every vector, scaled to an l1 norm below 1/2
+// so that no sum overflows.
+__device__ void vec_coefs(const VecHist* hist, int n, int s0, PoleState& s, int pole, int4* co, VecHead* head) {
+    double2 w = make_double2(0.0, 0.0), v = make_double2(1.0, 0.0);
+    double nw = 0.0, nv = 0.0;
+    for (int pass = 0; pass < 2; ++pass) {
+        double sw = 1.0, sv = 1.0;
+        if (pass == 1) {   // powers of two above twice the norms
+            if (nw > 0.0) sw = __hiloint2double(((__double2hiint(nw) >> 20) + 2) << 20, 0);
+            sv = __hiloint2double(((__double2hiint(nv) >> 20) + 2) << 20, 0);
+        }
+        for (int j = n - 1; j >= 0; --j) {
+            const VecHist h = hist[(size_t)j * kKryMaxPoles + pole];
+            const bool on = s.frz == 0 || s0 + 1 + j <= s.frz;
+            const double2 c = on ? h.c : make_double2(0.0, 0.0);
+            if (j == n - 1) {
+                w = c;
+                v = make_double2(1.0, 0.0);
+            } else {
+                w = make_double2(c.x - (h.m.x * w.x - h.m.y * w.y), c.y - (h.m.x * w.y + h.m.y * w.x));
+                v = make_double2(-(h.m.x * v.x - h.m.y * v.y), -(h.m.x * v.y + h.m.y * v.x));
+            }
+            if (pass == 0) {
+                nw += fabs(w.x) + fabs(w.y);
+                nv += fabs(v.x) + fabs(v.y);
+            } else {
+                const double f[4] = {w.x / sw, w.y / sw, v.x / sv, v.y / sv};
+                for (int k = 0; k < 4; ++k) {
+                    const int2 l = to_limbs(f[k]);
+                    co[4 * j + k] = make_int4(l.x, __float_as_int((float)l.x), __float_as_int((float)l.y), 0);
+                }
+            }
+        }
+        if (pass == 1) {
+            head->sw = sw;
+            head->sv = sv;
+            head->om = make_double2(-(s.mr * w.x - s.mi * w.y), -(s.mr * w.y + s.mi * w.x));
+            head->nu = make_double2(-(s.mr * v.x - s.mi * v.y), -(s.mr * v.y + s.mi * v.x));
+            head->act = s.frz == 0 || s.frz > s0;
+            head->first = s0 == 0;
+        }
+    }
+    const double2 m = hist[(size_t)(n - 1) * kKryMaxPoles + pole].m;
+    s.mr = m.x;
+    s.mi = m.y;
+}
+
+// x and p of one pole over the slab: fixed-point sums over the kept vectors
+// (the mixed terms in float, 2^-55 of the sum), joined in FP64.  A pair's
+// first point lies at X[xoff(item)], the second beside it.
+template <class F>
+__device__ __forceinline__ void vec_update(const SlabArgs& A, int n, const int4* co, const VecHead& h, const int4* Ub,
+                                           double2* X, double2* Pv, F&& xoff) {
+    const double sx = h.sw * 0x1p-62, sp = h.sv * 0x1p-62;
+    for (int item = threadIdx.x; item < A.n_items; item += blockDim.x) {
+        long long hh[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        const int4* up = Ub + item;
+#pragma unroll 2
+        for (int j = 0; j < n; ++j) {
+            const int4 u = *up;
+            up += A.n_items;
+            const float a0 = (float)u.x, b0 = (float)u.y, a1 = (float)u.z, b1 = (float)u.w;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int4 c = co[4 * j + k];
+                const float ch = __int_as_float(c.y), cl = __int_as_float(c.z);
+                madw(hh[2 * k], u.x, c.x);
+                madw(hh[2 * k + 1], u.z, c.x);
+                f[2 * k] = fmaf(a0, cl, fmaf(b0, ch, f[2 * k]));
+                f[2 * k + 1] = fmaf(a1, cl, fmaf(b1, ch, f[2 * k + 1]));
+            }
+        }
+        double2* x = X + xoff(item);
+        double2* p = Pv + 2 * (size_t)item;
+        const int pc = item % A.npc;
+        const int two = 2 * (pc % A.npx) + 1 < A.m0 ? 2 : 1;
+        for (int i = 0; i < two; ++i) {
+            double v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                v[k] = (double)((i ? hh[2 * k + 1] : hh[2 * k]) + (long long)((i ? f[2 * k + 1] : f[2 * k]) * 0x1p-31f));
+            double2 xv = make_double2(v[0] * sx, v[1] * sx), pv = make_double2(v[2] * sp, v[3] * sp);
+            if (!h.first) {
+                const double2 po = p[i], xo = x[i];
+                xv.x += xo.x + (h.om.x * po.x - h.om.y * po.y);
+                xv.y += xo.y + (h.om.x * po.y + h.om.y * po.x);
+                pv.x += h.nu.x * po.x - h.nu.y * po.y;
+                pv.y += h.nu.x * po.y + h.nu.y * po.x;
+            }
+            x[i] = xv;
+            p[i] = pv;
+        }
+    }
+}
+
 template <int Q, bool kNl>
 __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant__ KrylovParams P) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ KShared S;
+    __shared__ KSharedVec SV;
     __shared__ KSharedNl SN[1];   // untouched (and dropped) without projectors
     const uint64_t t_start = global_time_ns();
     const int C = (int)k_nrank(), rank = (int)k_rank();
@@ -659,7 +787,13 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
     char* slot = P.scratch + (size_t)blockIdx.x * P.cta_bytes;
     char* slot0 = P.scratch + (size_t)(blockIdx.x - rank) * P.cta_bytes;   // rank 0's slot
     int4* const Vp = reinterpret_cast<int4*>(slot);
-    int4* const Up = reinterpret_cast<int4*>(slot + P.off_up);
+    int4* const Up = reinterpret_cast<int4*>(slot + P.off_up);   // u_k limbs in place (k - 1) mod ring
+    const int ring = P.vec ? kKryVec : 1;
+    double2* const Xs = reinterpret_cast<double2*>(slot + P.off_x);
+    double2* const Ps = reinterpret_cast<double2*>(slot + P.off_p);
+    VecHist* const hist = reinterpret_cast<VecHist*>(slot0 + P.off_hist);
+    char* const coef = slot0 + P.off_coef;   // per pole: VecHead, then kKryVec x 4 int4
+    constexpr size_t kCoefBytes = 128 + sizeof(int4) * 4 * kKryVec;
     longlong2* const Wp = reinterpret_cast<longlong2*>(slot + P.off_w);
     uint4* const Rec = reinterpret_cast<uint4*>(slot + P.off_rec);
     KRow* const rows = reinterpret_cast<KRow*>(slot + P.off_rows);
@@ -710,7 +844,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 x[i] = split31(__double2ll_rn(v * vs));
             }
             Vp[t] = make_int4(x[0].x, x[0].y, x[1].x, x[1].y);
-            Up[t] = make_int4(0, 0, 0, 0);
+            Up[(size_t)(ring - 1) * n_items + t] = make_int4(0, 0, 0, 0);   // u_0 = 0
         }
         long long* acc = nullptr;   // [n_local][4] partial projections
         int2* cl = nullptr;         // [n_local][4] coefficients
@@ -759,7 +893,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
             __syncthreads();
             if (tid == 0) xtab[0] = ktab[0] = make_int4(0, 0, 0, 0);
         }
-        const SlabArgs SA{U, Vp, Up, Wp, Rec, m0, m1, npx, npc, n_items, pitch, pp,
+        const SlabArgs SA{U, Vp, Wp, Rec, m0, m1, npx, npc, n_items, pitch, pp,
                           make_fastdiv((uint32_t)npc), div_px};
         __syncthreads();
         // any CTA that cannot run the node stops the whole cluster
@@ -788,11 +922,57 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         if (scalar_warp && rank == 0 && P.K == 0) {
             for (int k = lane; k < P.P; k += 32, ++np) {
                 const double2 z = P.z[k];
-                ps[np] = PoleState{(z.x - P.shift) / P.scale, z.y / P.scale, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0, 1.0, 0};
+                ps[np] = PoleState{(z.x - P.shift) / P.scale, z.y / P.scale, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0, 1.0, 0, 0, 4.0, 0.0,
+                                   0.0, 0.0};
             }
         }
         k_sync();
 
+        // Where a pair's first point lies in a solution vector: region order in
+        // a checkpoint, pair order in scratch.
+        auto vec_index = [&](int item) -> long long {
+            if (!P.ckpt) return 2 * (long long)item;
+            const int d = (int)fdiv((uint32_t)item, SA.div_pc), pc = item - d * npc;
+            const int pb = (int)fdiv((uint32_t)pc, div_px);
+            return ((long long)(z0 + d) * m1 + pb) * m0 + 2 * (pc - pb * npx);
+        };
+        // Pole recurrences of step k (the scalar warp of rank 0); true once
+        // nothing is left to do.  x_jp(j) sums up to the step after the one
+        // at which all poles met tol, whether or not vectors are carried on.
+        int proc = 0, g_stop = 0;
+        bool all_done = false;
+        auto poles = [&](int step) {
+            bool all = true, done = true;
+            const double p2 = __hiloint2double((1023 + S.e_hat) << 20, 0);
+            for (int k = 0; k < np; ++k) {
+                PoleState& s = ps[k];
+                const double dr = S.a_hat - s.zr - s.er, di = -s.zi - s.ei;   // d of this step
+                pole_step(s, S.a_hat, S.b2_hat, g_stop == 0 || step <= g_stop);
+                if (P.vec) {
+                    const double inv = 1.0 / (dr * dr + di * di);
+                    VecHist h;
+                    h.c = make_double2((s.cr * dr + s.ci * di) * inv, (s.ci * dr - s.cr * di) * inv);
+                    h.m = make_double2(p2 * s.er, p2 * s.ei);
+                    hist[(size_t)((step - 1) % kKryVec) * kKryMaxPoles + lane + 32 * k] = h;
+                    s.cr = -h.c.x / p2;
+                    s.ci = -h.c.y / p2;
+                }
+                const double rn = sqrt(sqrt(s.fr * s.fr + s.fi * s.fi));
+                if (!s.conv) {
+                    s.rn = rn;
+                    if (rn <= P.tol) s.conv = step;
+                }
+                if (!s.frz && rn <= kFreeze * P.tol) s.frz = step;
+                all = all && s.conv;
+                done = done && s.frz;
+            }
+            all = __all_sync(0xffffffffu, all);
+            done = __all_sync(0xffffffffu, done);
+            if (all && !g_stop) g_stop = step + 1;
+            proc = step;
+            all_done = P.vec ? all && done : all;
+        };
+        int s0 = 0;   // steps the solution vectors hold
         int it = 0, stop = bad ? 1 : 0;
         while (!stop) {
             if constexpr (kNl) {
@@ -819,20 +999,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
             if (scalar_warp) {
                 // pole recurrences of the step before, while the others compute
                 if (rank == 0 && P.K == 0) {
-                    int flag = 0;
-                    if (it > 0) {
-                        bool all = true;
-                        for (int k = 0; k < np; ++k) {
-                            pole_step(ps[k], S.a_hat, S.b2_hat);
-                            const double r2 = sqrt(ps[k].fr * ps[k].fr + ps[k].fi * ps[k].fi);
-                            if (!ps[k].conv) {
-                                ps[k].rn = sqrt(r2);
-                                if (ps[k].rn <= P.tol) ps[k].conv = it;
-                            }
-                            all = all && ps[k].conv;
-                        }
-                        if (__all_sync(0xffffffffu, all)) flag = 1;
-                    }
+                    if (it > proc) poles(it);
+                    int flag = all_done ? 1 : 0;
                     if (P.timeout_ns && global_time_ns() - t_start > P.timeout_ns) flag = 2;
                     flag = __shfl_sync(0xffffffffu, flag, 0);
                     if (lane == 0) S.stop = flag;
@@ -841,9 +1009,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 }
             } else {
                 const int2 g = make_int2(-S.cg.x, -S.cg.y);
+                const int4* up = Up + (size_t)((it - 1 + ring) % ring) * n_items;
                 // (the compiler sees that these tables are in shared memory)
-                if (!kNl || tab_smem) slab_apply<Q, kNl>(P, SA, stab + n_x + 1, stab, nwp, g, hh1, l1, hh2, l2);
-                else slab_apply<Q, kNl>(P, SA, ktab, xtab, nwp, g, hh1, l1, hh2, l2);
+                if (!kNl || tab_smem) slab_apply<Q, kNl>(P, SA, stab + n_x + 1, stab, up, nwp, g, hh1, l1, hh2, l2);
+                else slab_apply<Q, kNl>(P, SA, ktab, xtab, up, nwp, g, hh1, l1, hh2, l2);
             }
             // ---- u.w and w.w over the cluster ------------------------------
             if (!scalar_warp) {
@@ -914,11 +1083,47 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                     S.stop = st;
                     S.a_hat = al;
                     S.b2_hat = b2;
+                    S.e_hat = e;
                     S.s0 = s0n;
                 }
             }
             __syncthreads();
             stop = S.stop;
+            if (P.vec && (stop || it % kKryVec == 0)) {
+                // apply the vectors kept to the solutions
+                const int n = it - s0;
+                if (scalar_warp && rank == 0) {
+                    if (it > proc) poles(it);
+                    __syncwarp();
+                    for (int k = 0; k < np; ++k) {
+                        char* cb = coef + (size_t)(lane + 32 * k) * kCoefBytes;
+                        vec_coefs(hist, n, s0, ps[k], lane + 32 * k, reinterpret_cast<int4*>(cb + 128),
+                                  reinterpret_cast<VecHead*>(cb));
+                    }
+                }
+                for (int item = tid; item < n_items; item += blockDim.x) {   // u_it itself
+                    const int d = (int)fdiv((uint32_t)item, SA.div_pc), pc = item - d * npc;
+                    const int pb = (int)fdiv((uint32_t)pc, div_px);
+                    Up[(size_t)((it - 1) % ring) * n_items + item] =
+                        *reinterpret_cast<const int4*>(U + (d + Q) * pp + pb * pitch + 2 * (pc - pb * npx));
+                }
+                k_sync();
+                for (int pole = 0; pole < P.P; ++pole) {
+                    const char* cb = coef + (size_t)pole * kCoefBytes;
+                    if (!__ldcg(reinterpret_cast<const int*>(cb + offsetof(VecHead, act)))) continue;
+                    __syncthreads();
+                    for (int t = tid; t < 4 * n; t += blockDim.x)
+                        SV.co[t] = __ldcg(reinterpret_cast<const int4*>(cb + 128) + t);
+                    if (tid < (int)(sizeof(VecHead) / 4))
+                        reinterpret_cast<int*>(&SV.head)[tid] = __ldcg(reinterpret_cast<const int*>(cb) + tid);
+                    __syncthreads();
+                    double2* x = P.ckpt ? P.ckpt + P.ckpt_off[(long long)node * P.P + pole]
+                                        : Xs + (size_t)pole * 2 * n_items;
+                    vec_update(SA, n, SV.co, SV.head, Up, x, Ps + (size_t)pole * 2 * n_items, vec_index);
+                }
+                s0 = it;
+                k_sync();   // from here the coefficients may be written again
+            }
             if (stop) break;
             if (scalar_warp) {
                 if (lane == 0) S.inv0 = 1.0 / S.s0;
@@ -949,7 +1154,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                         const long long t0 = w[j].x - fold(h0, g0), t1 = w[j].y - fold(h1, g1);
                         const int2 a = split31(e >= 0 ? t0 << e : t0 >> -e), b = split31(e >= 0 ? t1 << e : t1 >> -e);
                         const int4 nu = make_int4(a.x, a.y, b.x, b.y);
-                        Up[item] = u;
+                        Up[(size_t)((it - 1) % ring) * n_items + item] = u;
                         *up = nu;
                         // the CTAs whose halo holds this plane
                         const int z = z0 + d;
@@ -969,7 +1174,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         if (P.check && !bad) {
             double* c = reinterpret_cast<double*>(acc);   // free once the steps are done
             double* part = reinterpret_cast<double*>(cpart);
-            double s2 = check_step<Q, kNl>(P, SA, lo, z0, SN[0], c, S.cg_used, [&]() {
+            double s2 = check_step<Q, kNl>(P, SA, lo, z0, SN[0], c, Up + (size_t)((it - 2 + ring) % ring) * n_items, S.cg_used, [&]() {
                 __syncthreads();
                 for (int t = tid; t < n_loc4; t += blockDim.x) part[t] = c[t];
                 k_sync();
@@ -993,8 +1198,43 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
             for (int r = 0; r < C; ++r) defect += __longlong_as_double(S.mbox[r][0]);
             defect = sqrt(defect * S.inv0) * P.scale;   // relative to ||u||, in units of H
         }
+        // ---- outputs of the solution vectors ----------------------------------
+        if (P.vec) {
+            if (tid < P.P) {
+                const double2 z = P.z[tid], w = P.w[tid];
+                const double aj = P.fused_a ? P.fused_a[node] : 0.0, bj = P.fused_b ? P.fused_b[node] : 0.0;
+                const double cr = 2.0 * aj / P.dV + 2.0 * bj * z.x, ci = 2.0 * bj * z.y;
+                SV.cp[tid] = P.dm_rows ? w : make_double2(cr * w.x - ci * w.y, cr * w.y + ci * w.x);
+            }
+            __syncthreads();
+            const double inv = 1.0 / P.scale, nan = __longlong_as_double(0x7ff8000000000000LL);
+            for (int item = tid; item < n_items; item += blockDim.x) {
+                const int d = (int)fdiv((uint32_t)item, SA.div_pc), pc = item - d * npc;
+                const int pb = (int)fdiv((uint32_t)pc, div_px), a = 2 * (pc - pb * npx);
+                const long long xi = vec_index(item);
+                for (int i = 0; i < 2 && a + i < m0; ++i) {
+                    double sum = 0.0;
+                    for (int pole = 0; pole < P.P; ++pole) {
+                        double2* xp = (P.ckpt ? P.ckpt + P.ckpt_off[(long long)node * P.P + pole]
+                                              : Xs + (size_t)pole * 2 * n_items) + xi + i;
+                        const double2 x = bad ? make_double2(nan, nan) : make_double2(xp->x * inv, xp->y * inv);
+                        if (P.ckpt) *xp = x;
+                        const double2 c = SV.cp[pole];
+                        if (P.dm_rows) sum += c.x * x.y + c.y * x.x;
+                        else sum -= c.x * (2.0 * x.x * x.y) + c.y * (x.x * x.x - x.y * x.y);
+                    }
+                    if (P.dm_rows) P.dm_rows[P.dm_off[node] + ((long long)(z0 + d) * m1 + pb) * m0 + a + i] = sum;
+                    if (P.fused_dLdV) {
+                        const int gx = wrap_once(lo[0] + a + i, P.n[0]), gy = wrap_once(lo[1] + pb, P.n[1]);
+                        const int gz = wrap_once(lo[2] + z0 + d, P.n[2]);
+                        atomicAdd(P.fused_dLdV + gx + (long long)P.n[0] * (gy + (long long)P.n[1] * gz), sum);
+                    }
+                }
+            }
+        }
         // ---- results ---------------------------------------------------------
         if (rank == 0 && scalar_warp) {
+            if (P.K == 0 && it > proc) poles(it);
             if (P.K > 0) {
                 if (lane == 0) {
                     P.k_used[node] = bad ? 0 : it;
@@ -1002,13 +1242,6 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 }
             } else {
                 for (int k = 0; k < np; ++k) {
-                    if (!bad && it > 0) {
-                        pole_step(ps[k], S.a_hat, S.b2_hat);
-                        if (!ps[k].conv) {
-                            ps[k].rn = sqrt(sqrt(ps[k].fr * ps[k].fr + ps[k].fi * ps[k].fi));
-                            if (ps[k].rn <= P.tol) ps[k].conv = it;
-                        }
-                    }
                     const long long o = (long long)node * P.P + lane + 32 * k;
                     const double nan = __longlong_as_double(0x7ff8000000000000LL);
                     // the true residual: the recurrence's and, with ||x||^2 =
@@ -1117,7 +1350,10 @@ cudaError_t launch(const KrylovParams& P, int csz, int grid, int block, size_t s
 size_t kry_u_bytes(int q, int m0, int m1, int depth) {
     return ((size_t)(depth + 2 * q) * kry_pitch(q, m0) * m1 * sizeof(int2) + 15) / 16 * 16;
 }
-size_t kry_static_smem_bytes(int) { return sizeof(KShared) + sizeof(KSharedNl) + 64; }
+size_t kry_static_smem_bytes(int) { return sizeof(KShared) + sizeof(KSharedNl) + sizeof(KSharedVec) + 64; }
+size_t kry_vec_bytes(int P) {
+    return (size_t)kKryVec * kKryMaxPoles * sizeof(VecHist) + (size_t)P * (128 + 64 * kKryVec);
+}
 int kry_max_threads() { return kMaxThreads - 32; }
 
 int kry_max_clusters(int q, int nonlocal, int csz, int block, size_t smem) {

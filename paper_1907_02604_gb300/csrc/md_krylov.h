@@ -15,6 +15,7 @@ namespace md {
 constexpr int kKryMaxQ = 4;        // stencil half-widths 1..4 (fd_order <= 8)
 constexpr int kKryMaxPoles = 64;
 constexpr int kKryChunkRows = 32;  // projector rows of one atom a warp sums in one go
+constexpr int kKryVec = 32;        // Krylov vectors kept between two updates of the solution vectors
 constexpr int kKryMaxDepth = 40;   // planes of a CTA's slab (bounds the exact partial sums)
 
 struct KrylovParams {
@@ -63,6 +64,18 @@ struct KrylovParams {
     int* iters;
     double* resid;
     int* n_rel;
+    // Solution vectors: with vec, x_jp is accumulated over the region (in ckpt,
+    // or in scratch) and used for the outputs below
+    int vec;
+    size_t off_x, off_p, off_hist, off_coef;
+    double2* ckpt;                 // NULL or checkpoint base
+    const long long* ckpt_off;     // point offset of system (node*P + pole) in ckpt
+    double* fused_dLdV;            // fused adjoint, see SolveParams
+    const double* fused_a;
+    const double* fused_b;
+    const double2* w;
+    double* dm_rows;
+    const long long* dm_off;
     // Lanczos rules: K > 0 stops after K steps and stores the coefficients
     int K;
     double breakdown_tol;
@@ -77,6 +90,8 @@ struct KrylovParams {
 // dynamic shared memory).
 size_t kry_u_bytes(int q, int m0, int m1, int depth);
 size_t kry_static_smem_bytes(int nonlocal);
+// Scratch of the solution vectors' coefficients, per CTA.
+size_t kry_vec_bytes(int P);
 int kry_max_threads();
 // Resident clusters of csz CTAs; 0 if the shape cannot run.
 int kry_max_clusters(int q, int nonlocal, int csz, int block, size_t smem);
