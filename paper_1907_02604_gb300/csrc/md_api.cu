@@ -245,7 +245,7 @@ namespace {
 // ---------------------------------------------------------------------------
 
 constexpr int kKryClasses = 12;   // region-size classes of one batch, launched side by side
-constexpr int kKryStreams = 4;    // the caller's stream and the three of KrySide
+constexpr int kKryStreams = 12;   // the caller's stream and those of KrySide: a class to each
 
 }  // namespace
 
@@ -257,8 +257,9 @@ struct KryClass {
 
 // Side streams of a launch of several classes.
 struct KrySide {
-    cudaStream_t s[3] = {};
-    cudaEvent_t fork = nullptr, join[3] = {};
+    cudaStream_t s[11] = {};
+    cudaEvent_t fork = nullptr, join[11] = {};
+    int n = 0;
 };
 
 namespace {
@@ -282,7 +283,8 @@ void kry_operator(KrylovParams& P, const Ham& H, double scale) {
             const long long x = o < H.q ? std::llrint(std::ldexp(H.coef[d][o] / scale, 62)) : 0;
             const long long hi = (x + (1LL << 30)) >> 31;
             P.wh[d][o] = (int)hi;
-            P.wl[d][o] = (int)(x - (hi << 31));
+            const float f[2] = {(float)(x - (hi << 31)), (float)hi};
+            std::memcpy(&P.wf[d][o], f, sizeof(f));
         }
 }
 
@@ -329,9 +331,9 @@ KryShape kry_shape(const Ham& H, int m0, int m1, int m2, int c, int dev) {
                                               std::min<double>(H.n_atoms, kMaxLocalProjAtoms));
         const double here = std::min(local, per_pt * reach[0] * reach[1] * reach[2]);
         const double rows = here * 3.2 * H.proj_rc * H.proj_rc / (H.h[1] * H.h[2]) * m1 / reach[1] * s.depth / reach[2];
-        tables = (size_t)(kry_max_threads() * 32 + 1024 + local * 96);
+        tables = (size_t)(local * 96);
         if (u + kry_max_threads() * 32 + 1024 > budget) return s;
-        s.spill = u + tables + (size_t)(1.15 * (rows + here * 2.0 * H.proj_rc / H.h[0]) * 16) > budget;
+        s.spill = u + tables + (size_t)((std::max(1.1 * rows, 1280.0) + 1.1 * here * (2.0 * H.proj_rc / H.h[0] + 2)) * 16) > budget;
     } else if (u > budget) {
         return s;
     }
@@ -509,14 +511,13 @@ void kry_scratch(std::vector<KryClass>& cls, char* base, const int* list, unsign
     }
 }
 
-cudaError_t kry_side_create(KrySide& d) {
-    if (d.fork) return cudaSuccess;
-    for (int i = 0; i < kKryStreams - 1; ++i) {
-        cudaError_t e = cudaStreamCreateWithFlags(&d.s[i], cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&d.join[i], cudaEventDisableTiming);
+cudaError_t kry_side_create(KrySide& d, int n) {
+    for (; d.n < n; ++d.n) {
+        cudaError_t e = cudaStreamCreateWithFlags(&d.s[d.n], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&d.join[d.n], cudaEventDisableTiming);
         if (e != cudaSuccess) return e;
     }
-    return cudaEventCreateWithFlags(&d.fork, cudaEventDisableTiming);
+    return d.fork ? cudaSuccess : cudaEventCreateWithFlags(&d.fork, cudaEventDisableTiming);
 }
 
 void kry_side_free(KrySide& d) {
@@ -536,7 +537,7 @@ cudaError_t kry_launch(const std::vector<KryClass>& cls, const Ham& H, KrySide& 
     const int ns = std::min<int>(kKryStreams, (int)cls.size());
     cudaError_t e = cudaSuccess;
     if (ns > 1) {
-        e = kry_side_create(side);
+        e = kry_side_create(side, ns - 1);
         if (e == cudaSuccess) e = cudaEventRecord(side.fork, stream);
         for (int i = 1; i < ns && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(side.s[i - 1], side.fork, 0);
     }
@@ -911,7 +912,7 @@ cudaError_t plan_capture(md_plan* pl) {
     pl->exec = nullptr;
     pl->graph = nullptr;
     if (pl->kry.size() > 1) {   // made outside the capture
-        const cudaError_t e = kry_side_create(pl->side);
+        const cudaError_t e = kry_side_create(pl->side, std::min<int>(kKryStreams, (int)pl->kry.size()) - 1);
         if (e != cudaSuccess) return e;
     }
     cudaError_t e = cudaStreamBeginCapture(pl->cap, cudaStreamCaptureModeThreadLocal);

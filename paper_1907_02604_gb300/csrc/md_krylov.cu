@@ -105,50 +105,82 @@ __device__ __forceinline__ int opaque(int x) {
     asm("" : "+r"(x));
     return x;
 }
-__device__ __forceinline__ int4 opaque(int4 v) { return make_int4(opaque(v.x), opaque(v.y), opaque(v.z), opaque(v.w)); }
 __device__ __forceinline__ int2 split31(long long x) {
     x += 1LL << 30;
     return make_int2(opaque((int)(x >> 31)), opaque((int)(x & 0x7fffffffLL) - (1 << 30)));
 }
-// (hh, hl) += a * b
-__device__ __forceinline__ void mac(long long& hh, long long& hl, int ah, int al, int bh, int bl) {
-    madw(hh, ah, bh);
-    madw(hl, ah, bl);
-    madw(hl, al, bh);
+// A product of two 62-bit values is hi hi 2^-62 + (hi lo + lo hi) 2^-93 + ..:
+// the first term exactly, in 64 bits; the mixed terms, 2^-31 of it, in FP32
+// (2^-55 of the product, FP64's own rounding is 2^-54).  IMAD.WIDE with
+// distinct operands runs at 31 a clock and SM (measured), FFMA2 at 65 pairs,
+// so the mixed terms cost a quarter of what they did in 64-bit integers.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
 }
-// the same with the mixed terms in two sums: half the chain of dependent additions
-__device__ __forceinline__ void mac2(long long& hh, long long& hl, long long& hm, int ah, int al, int bh, int bl) {
-    madw(hh, ah, bh);
-    madw(hl, ah, bl);
-    madw(hm, al, bh);
+__device__ __forceinline__ float sum2(f32x2 v) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return a + b;
 }
-// Partial sums of u.w and w.w: hi hi exact, the mixed terms in 64 bits, the
-// lo lo terms (which in w.w add up: 2e-13 of the sum if left out) in float.
-__device__ __forceinline__ void dots(int2 u, int2 w, long long& hh1, long long& x1, long long& y1, long long& hh2,
-                                     long long& x2, float& q1, float& q2) {
-    madw(hh1, u.x, w.x);
-    madw(x1, u.x, w.y);
-    madw(y1, u.y, w.x);
-    madw(hh2, w.x, w.x);
-    madw(x2, w.x, w.y);
-    const float f = (float)w.y;
-    q1 = fmaf((float)u.y, f, q1);
-    q2 = fmaf(f, f, q2);
+// acc += a b, elementwise
+__device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
-constexpr long long kHalf = 1LL << 30;   // start of hl: rounds the result to nearest
-__device__ __forceinline__ long long fold(long long hh, long long hl) { return hh + (hl >> 31); }
+struct Acc {
+    long long hh = 0;
+    f32x2 f = 0;      // mixed terms, units of 2^-93
+    float s = 0.f;    // those of table entries
+    // += (ah, af) * (bh, bf), af = {(float)hi, (float)lo}, bf = {(float)lo, (float)hi}
+    __device__ __forceinline__ void mac(int ah, f32x2 af, int bh, f32x2 bf) {
+        madw(hh, ah, bh);
+        fma2(f, af, bf);
+    }
+    // += (ah, (float)ah, al) * (bh, (float)bh, bl)
+    __device__ __forceinline__ void mac(int ah, float af, float al, int bh, float bf, float bl) {
+        madw(hh, ah, bh);
+        s = fmaf(af, bl, fmaf(al, bf, s));
+    }
+    // rounded to 2^-62; |mixed| < 2^62, as ||u|| < 1/4
+    __device__ __forceinline__ long long fold() const { return hh + __float2int_rn((sum2(f) + s) * 0x1p-31f); }
+};
+__device__ __forceinline__ f32x2 hi_lo(int h, int l) { return pack((float)h, (float)l); }
+__device__ __forceinline__ f32x2 lo_hi(int h, int l) { return pack((float)l, (float)h); }
+// A table entry (hi, bits of (float)lo) as operand; a pair in registers would
+// have to be assembled by moves, so these mixed terms are single FMAs.
+struct TabVal {
+    int h;
+    float f, l;
+};
+__device__ __forceinline__ TabVal tv(int hi, int lo) { return TabVal{hi, (float)hi, __int_as_float(lo)}; }
+__device__ __forceinline__ void tmac(Acc& a, const TabVal& x, const TabVal& y) { a.mac(x.h, x.f, x.l, y.h, y.f, y.l); }
+__device__ __forceinline__ int2 tab_limbs(int2 v) { return make_int2(v.x, __float_as_int((float)v.y)); }
+// Partial sums of u.w and w.w: hi hi exact, the rest in float (lo lo terms
+// included: in w.w they add up, 2e-13 of the sum).
+struct Dots {
+    long long hh1 = 0, hh2 = 0;
+    f32x2 f1 = 0, f2 = 0;
+    float q1 = 0.f;
+    __device__ __forceinline__ void add(int uh, f32x2 uf, int2 w) {
+        madw(hh1, uh, w.x);
+        madw(hh2, w.x, w.x);
+        const float wh = (float)w.x, wl = (float)w.y;
+        fma2(f1, uf, pack(wl, wh));
+        fma2(f2, pack(wh, wl), pack(wl, wl * 0x1p-32f));
+        q1 = fmaf(__uint_as_float((uint32_t)(uf >> 32)), wl * 0x1p-31f, q1);
+    }
+    // mixed parts in units of 2^-83 (w.w: half of them)
+    __device__ __forceinline__ long long l1() const { return __float2ll_rn((sum2(f1) + q1) * 0x1p-10f); }
+    __device__ __forceinline__ long long l2() const { return __float2ll_rn(sum2(f2) * 0x1p-10f); }
+};
 __device__ __forceinline__ int2 to_limbs(double v) { return split31(__double2ll_rn(v * 0x1p62)); }
-
-__device__ __forceinline__ long long warp_sum_i(long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 
 struct KRow {        // one run of a projector row inside the slab
     int voff;        // index of window slot 0 in the u buffer
     int uu;          // u0 | u1 << 8 | local atom << 16
-    int2 r0, r1, r2; // g_y g_z, (d g)_y g_z, g_y (d g)_z
+    int2 r0, r1, r2; // g_y g_z, (d g)_y g_z, g_y (d g)_z: hi, (float)lo
 };
 static_assert(sizeof(KRow) == 32, "row record");
 
@@ -159,7 +191,7 @@ struct KChunk {      // up to kKryChunkRows rows of one atom
 struct KShared {
     long long part[kMaxWarps][4];
     long long mbox[kMaxC][5];     // per rank: u.w (2), w.w (2), stop flag of rank 0
-    int2 ca, cg, cg_used;         // alpha and g as limbs; the g of the step in hand
+    int2 ca, cg;                  // alpha and g as limbs
     int e;                        // u_new = (w - alpha u) 2^e
     int zlo[kMaxC + 1];           // first plane of each rank's slab
     int stop;                     // 0, 1 done, 2 timeout
@@ -277,15 +309,13 @@ __device__ void build_rows(const KrylovParams& P, const int m[3], const int lo[3
                     r.voff = (c - z0 + q) * pp + b * pitch + sh;
                     r.uu = u0 | (u1 << 8) | (k << 16);
                     const int4 y = ty[vv], z = tz[ww];
-                    long long hh = 0, hl = kHalf;
-                    mac(hh, hl, y.x, y.y, z.x, z.y);
-                    r.r0 = split31(fold(hh, hl));
-                    hh = 0, hl = kHalf;
-                    mac(hh, hl, y.z, y.w, z.x, z.y);
-                    r.r1 = split31(fold(hh, hl));
-                    hh = 0, hl = kHalf;
-                    mac(hh, hl, y.x, y.y, z.z, z.w);
-                    r.r2 = split31(fold(hh, hl));
+                    Acc r0, r1, r2;
+                    tmac(r0, tv(y.x, y.y), tv(z.x, z.y));
+                    tmac(r1, tv(y.z, y.w), tv(z.x, z.y));
+                    tmac(r2, tv(y.x, y.y), tv(z.z, z.w));
+                    r.r0 = tab_limbs(split31(r0.fold()));
+                    r.r1 = tab_limbs(split31(r1.fold()));
+                    r.r2 = tab_limbs(split31(r2.fold()));
                     rows[id] = r;
                     const int item0 = ((c - z0) * m[1] + b) * npx;
                     for (int pr = (u0 + sh) >> 1; pr <= (u1 + sh) >> 1; ++pr) {
@@ -375,7 +405,7 @@ __device__ __forceinline__ void project(const KrylovParams& P, const int2* __res
         long long s0 = 0, s1 = 0, s2 = 0, s3 = 0;
         for (int ub = 0; ub < P.win_x; ub += 16) {
             const int u = ub + (lane & 15);
-            long long ah = 0, al = kHalf, bh = 0, bl = kHalf, ch_ = 0, cl_ = kHalf;
+            Acc A0, A1, A2;
             const int4* st = stage + 2 * half;
             // rows past the count are empty runs, so the half warps stay together
 #pragma unroll 4
@@ -385,25 +415,24 @@ __device__ __forceinline__ void project(const KrylovParams& P, const int2* __res
                 int2 v = make_int2(0, 0);
                 if (u >= u0 && u <= u1) v = U[a.x + u];
                 v.x = opaque(v.x);
-                v.y = opaque(v.y);
-                mac(ah, al, v.x, v.y, a.z, a.w);
-                mac(bh, bl, v.x, v.y, b.x, b.y);
-                mac(ch_, cl_, v.x, v.y, b.z, b.w);
+                const float vh = (float)v.x, vl = (float)v.y;
+                A0.mac(v.x, vh, vl, a.z, (float)a.z, __int_as_float(a.w));
+                A1.mac(v.x, vh, vl, b.x, (float)b.x, __int_as_float(b.y));
+                A2.mac(v.x, vh, vl, b.z, (float)b.z, __int_as_float(b.w));
             }
             const int4 t = u < P.win_x ? xtab[k.tab + u] : make_int4(0, 0, 0, 0);
-            const int2 A = split31(fold(ah, al)), B = split31(fold(bh, bl)), D = split31(fold(ch_, cl_));
-            long long hh = 0, hl = kHalf;
-            mac(hh, hl, A.x, A.y, t.x, t.y);
-            s0 += fold(hh, hl);
-            hh = 0, hl = kHalf;
-            mac(hh, hl, A.x, A.y, t.z, t.w);
-            s1 += fold(hh, hl);
-            hh = 0, hl = kHalf;
-            mac(hh, hl, B.x, B.y, t.x, t.y);
-            s2 += fold(hh, hl);
-            hh = 0, hl = kHalf;
-            mac(hh, hl, D.x, D.y, t.x, t.y);
-            s3 += fold(hh, hl);
+            const TabVal g = tv(t.x, t.y), dg = tv(t.z, t.w);
+            const int2 l0 = tab_limbs(split31(A0.fold())), l1 = tab_limbs(split31(A1.fold()));
+            const int2 l2 = tab_limbs(split31(A2.fold()));
+            Acc r0, r1, r2, r3;
+            tmac(r0, tv(l0.x, l0.y), g);
+            tmac(r1, tv(l0.x, l0.y), dg);
+            tmac(r2, tv(l1.x, l1.y), g);
+            tmac(r3, tv(l2.x, l2.y), g);
+            s0 += r0.fold();
+            s1 += r1.fold();
+            s2 += r2.fold();
+            s3 += r3.fold();
         }
         const long long s = warp_sum4(s0, s1, s2, s3, lane);
         if (lane < 4)
@@ -417,15 +446,13 @@ __device__ __forceinline__ int4 row_factors(const KRow* row, const int2* cl) {
     const int4 a = reinterpret_cast<const int4*>(row)[0], b = reinterpret_cast<const int4*>(row)[1];
     const int4* c = reinterpret_cast<const int4*>(cl + 4 * ((a.y >> 16) & 0xff));
     const int4 c01 = c[0], c23 = c[1];
-    long long hh = 0, hl = kHalf;
-    mac(hh, hl, a.z, a.w, c01.x, c01.y);
-    mac(hh, hl, b.x, b.y, c23.x, c23.y);
-    mac(hh, hl, b.z, b.w, c23.z, c23.w);
-    const int2 k1 = split31(fold(hh, hl));
-    hh = 0, hl = kHalf;
-    mac(hh, hl, a.z, a.w, c01.z, c01.w);
-    const int2 k2 = split31(fold(hh, hl));
-    return make_int4(k1.x, k1.y, k2.x, k2.y);
+    Acc k1, k2;
+    tmac(k1, tv(a.z, a.w), tv(c01.x, c01.y));
+    tmac(k1, tv(b.x, b.y), tv(c23.x, c23.y));
+    tmac(k1, tv(b.z, b.w), tv(c23.z, c23.w));
+    tmac(k2, tv(a.z, a.w), tv(c01.z, c01.w));
+    const int2 x = tab_limbs(split31(k1.fold())), y = tab_limbs(split31(k2.fold()));
+    return make_int4(x.x, x.y, y.x, y.y);
 }
 
 // A slab as pairs of points (2k, 2k+1) along x, `npc` a plane: two points a
@@ -441,22 +468,23 @@ struct SlabArgs {
 };
 
 // Nonlocal term of one record entry on both points of a pair.
-__device__ __forceinline__ void nl_entry(const int4* ktab, const int4* xtab, uint32_t e0, uint32_t e1,
-                                         long long (&hh)[2], long long (&hl)[2], long long (&hm)[2]) {
+__device__ __forceinline__ void nl_entry(const int4* ktab, const int4* xtab, uint32_t e0, uint32_t e1, Acc (&acc)[2]) {
     const int4 k = ktab[e0 & 0xffffu], t0 = xtab[e0 >> 16], t1 = xtab[e1];
-    mac2(hh[0], hl[0], hm[0], t0.x, t0.y, k.x, k.y);
-    mac2(hh[1], hl[1], hm[1], t1.x, t1.y, k.x, k.y);
-    mac2(hh[0], hl[0], hm[0], t0.z, t0.w, k.z, k.w);
-    mac2(hh[1], hl[1], hm[1], t1.z, t1.w, k.z, k.w);
+    const TabVal k1 = tv(k.x, k.y), k2 = tv(k.z, k.w);
+    tmac(acc[0], tv(t0.x, t0.y), k1);
+    tmac(acc[1], tv(t1.x, t1.y), k1);
+    tmac(acc[0], tv(t0.z, t0.w), k2);
+    tmac(acc[1], tv(t1.z, t1.w), k2);
 }
 
 // Sums of the stencil's off-diagonal terms on a pair at p (16-byte units);
 // kInside: the rows b-Q .. b+Q all lie in the region.
 template <int Q, bool kInside>
 __device__ __forceinline__ void stencil(const KrylovParams& P, const SlabArgs& A, const int4* p, int4 c, int a, int b,
-                                        long long (&hh)[2], long long (&hl)[2], long long (&hm)[2]) {
+                                        Acc (&acc)[2]) {
     constexpr int H = (Q + 1) / 2;   // loads on either side of the pair
     const int pitch = A.pitch >> 1, pp = A.pp >> 1;
+    auto add = [&](int i, int h, int l, int d, int o) { acc[i].mac(h, hi_lo(h, l), P.wh[d][o - 1], P.wf[d][o - 1]); };
     {
         int2 x[2 * (2 * H + 1)];     // the row around the pair: x[2H], x[2H+1] are its points
 #pragma unroll
@@ -470,21 +498,21 @@ __device__ __forceinline__ void stencil(const KrylovParams& P, const SlabArgs& A
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 const int2 xa = x[2 * H + i + o], xb = x[2 * H + i - o];
-                mac2(hh[i], hl[i], hm[i], xa.x + xb.x, xa.y + xb.y, P.wh[0][o - 1], P.wl[0][o - 1]);
+                add(i, xa.x + xb.x, xa.y + xb.y, 0, o);
             }
     }
     const int zero = (((A.m0 + 1) & ~1) - a) >> 1;   // two of the zeros after this row
 #pragma unroll
     for (int o = 1; o <= Q; ++o) {
         const int4 ya = p[kInside || b + o < A.m1 ? o * pitch : zero], yb = p[kInside || b - o >= 0 ? -o * pitch : zero];
-        mac2(hh[0], hl[0], hm[0], ya.x + yb.x, ya.y + yb.y, P.wh[1][o - 1], P.wl[1][o - 1]);
-        mac2(hh[1], hl[1], hm[1], ya.z + yb.z, ya.w + yb.w, P.wh[1][o - 1], P.wl[1][o - 1]);
+        add(0, ya.x + yb.x, ya.y + yb.y, 1, o);
+        add(1, ya.z + yb.z, ya.w + yb.w, 1, o);
     }
 #pragma unroll
     for (int o = 1; o <= Q; ++o) {
         const int4 za = p[o * pp], zb = p[-o * pp];
-        mac2(hh[0], hl[0], hm[0], za.x + zb.x, za.y + zb.y, P.wh[2][o - 1], P.wl[2][o - 1]);
-        mac2(hh[1], hl[1], hm[1], za.z + zb.z, za.w + zb.w, P.wh[2][o - 1], P.wl[2][o - 1]);
+        add(0, za.x + zb.x, za.y + zb.y, 2, o);
+        add(1, za.z + zb.z, za.w + zb.w, 2, o);
     }
 }
 
@@ -495,55 +523,46 @@ __device__ __forceinline__ void stencil(const KrylovParams& P, const SlabArgs& A
 // and 19 warps at 96 registers are the faster trade.
 template <int Q, bool kNl>
 __device__ __forceinline__ void slab_apply(const KrylovParams& P, const SlabArgs& A, const int4* ktab,
-                                           const int4* xtab, const int4* u_prev, int nw, int2 g, long long& hh1,
-                                           long long& l1, long long& hh2, long long& l2) {
-    long long x1 = 0, y1 = 0, x2 = 0;
-    float q1 = 0.f, q2 = 0.f;
-    int steps = 0;
+                                           const int4* xtab, const int4* u_prev, int nw, int2 g, Dots& dots) {
+    const f32x2 gf = lo_hi(g.x, g.y);
     // lanes past the last pair repeat it and add nothing, so that warps stay whole
     for (int i0 = threadIdx.x & ~31; i0 < A.n_items; i0 += 32 * nw) {
         const int i = i0 + (int)(threadIdx.x & 31);
         const bool act = i < A.n_items;
         const int item = act ? i : A.n_items - 1;
-        const int4 v = A.Vp[item], um = u_prev[item];   // from L2, used after the stencil sums
+        const int4 v = A.Vp[item], um = u_prev[item];   // used after the stencil sums
         uint4 rc = make_uint4(0u, 0u, 0u, 0u);
         if (kNl) rc = A.Rec[(size_t)item * P.rec_words];
         const int d = (int)fdiv((uint32_t)item, A.div_pc), pc = item - d * A.npc;
         const int b = (int)fdiv((uint32_t)pc, A.div_px), a = 2 * (pc - b * A.npx);
         const int4* p = reinterpret_cast<const int4*>(A.U + (d + Q) * A.pp + b * A.pitch + a);
         const int4 c = *p;
-        long long hh[2] = {0, 0}, hl[2] = {kHalf, kHalf}, hm[2] = {0, 0};
-        if (__all_sync(0xffffffffu, b >= Q && b + Q < A.m1)) stencil<Q, true>(P, A, p, c, a, b, hh, hl, hm);
-        else stencil<Q, false>(P, A, p, c, a, b, hh, hl, hm);
-        mac2(hh[0], hl[0], hm[0], c.x, c.y, v.x, v.y);
-        mac2(hh[1], hl[1], hm[1], c.z, c.w, v.z, v.w);
-        const int gx = opaque(g.x), gy = opaque(g.y);
-        mac2(hh[0], hl[0], hm[0], um.x, um.y, gx, gy);
-        mac2(hh[1], hl[1], hm[1], um.z, um.w, gx, gy);
+        Acc acc[2];
+        if (__all_sync(0xffffffffu, b >= Q && b + Q < A.m1)) stencil<Q, true>(P, A, p, c, a, b, acc);
+        else stencil<Q, false>(P, A, p, c, a, b, acc);
+        const f32x2 c0 = hi_lo(c.x, c.y), c1 = hi_lo(c.z, c.w);
+        acc[0].mac(c.x, c0, v.x, lo_hi(v.x, v.y));
+        acc[1].mac(c.z, c1, v.z, lo_hi(v.z, v.w));
+        const int gx = opaque(g.x);
+        acc[0].mac(um.x, hi_lo(um.x, um.y), gx, gf);
+        acc[1].mac(um.z, hi_lo(um.z, um.w), gx, gf);
         if constexpr (kNl) {
             for (int q = 0; q < P.rec_words; ++q) {
                 const uint4 r = q == 0 ? rc : A.Rec[(size_t)item * P.rec_words + q];
                 if (!__any_sync(0xffffffffu, r.x)) break;
-                nl_entry(ktab, xtab, r.x, r.y, hh, hl, hm);
+                nl_entry(ktab, xtab, r.x, r.y, acc);
                 if (!__any_sync(0xffffffffu, r.z)) break;
-                nl_entry(ktab, xtab, r.z, r.w, hh, hl, hm);
+                nl_entry(ktab, xtab, r.z, r.w, acc);
             }
         }
-        const long long r0 = fold(hh[0], hl[0] + hm[0]);
-        const long long r1 = a + 1 < A.m0 ? fold(hh[1], hl[1] + hm[1]) : 0;
+        const long long r0 = acc[0].fold();
+        const long long r1 = a + 1 < A.m0 ? acc[1].fold() : 0;
         if (act) {
             A.Wp[item] = make_longlong2(r0, r1);
-            dots(make_int2(c.x, c.y), split31(r0), hh1, x1, y1, hh2, x2, q1, q2);
-            dots(make_int2(c.z, c.w), split31(r1), hh1, x1, y1, hh2, x2, q1, q2);
-        }
-        if ((++steps & 7) == 0) {   // 16 points: the mixed sums stay below 2^62.5
-            l1 += (x1 >> 10) + (y1 >> 10);
-            l2 += x2 >> 10;
-            x1 = y1 = x2 = 0;
+            dots.add(c.x, c0, split31(r0));
+            dots.add(c.z, c1, split31(r1));
         }
     }
-    l1 += (x1 >> 10) + (y1 >> 10) + (long long)(q1 * 0x1p-41f);
-    l2 += (x2 >> 10) + (long long)(q2 * 0x1p-42f);
 }
 
 __device__ __forceinline__ double limbs(int hi, int lo) { return fma((double)hi, 0x1p-31, (double)lo * 0x1p-62); }
@@ -852,7 +871,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         int4* xtab = nullptr;       // x tables of the slab's atoms
         int4* ktab = nullptr;       // [1 + n_rows] row factors of the apply, a zero row first
         bool tab_smem = true;       // both in shared memory
-        int4* stab = nullptr;       // where the tables lie in shared memory
+        int4 *xt_s = nullptr, *kt_s = nullptr;   // where they lie in shared memory
         int4* stage = nullptr;      // rows of the chunk a warp works on
         const KChunk* chk = chunks;
         int n_loc4 = 0, n_rows = 0, n_x = 0;
@@ -864,22 +883,25 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
             n_rows = min(SN[0].n_rows, P.row_cap);
             n_x = SN[0].n_tab * P.win_x;
             const size_t off = ((size_t)(depth + 2 * Q) * pp * sizeof(int2) + 15) / 16 * 16;
-            stage = reinterpret_cast<int4*>(dsm + off);
-            acc = reinterpret_cast<long long*>(stage + (nwp + 1) * 2 * kKryChunkRows);
+            // [projections][x tables][chunks][row factors | staged rows]: the
+            // rows are staged before the factors are formed
+            acc = reinterpret_cast<long long*>(dsm + off);
             cl = reinterpret_cast<int2*>(acc + n_loc4);
             cf = reinterpret_cast<double*>(cl + n_loc4);
-            stab = reinterpret_cast<int4*>(cf + n_loc4);
+            xt_s = reinterpret_cast<int4*>(cf + n_loc4);
             int4* const xg = reinterpret_cast<int4*>(slot + P.off_xtab);
-            const int n_ch = SN[0].n_chunks;
-            if ((size_t)((unsigned char*)stab - dsm) + (size_t)(n_x + n_rows + n_ch + 2) * 16 <= (size_t)P.smem_bytes) {
-                xtab = stab;
-                ktab = xtab + n_x + 1;
-                KChunk* cs = reinterpret_cast<KChunk*>(ktab + n_rows + 1);
+            const int n_ch = SN[0].n_chunks, n_st = (nwp + 1) * 2 * kKryChunkRows;
+            kt_s = xt_s + n_x + 1 + n_ch;
+            if ((size_t)((unsigned char*)kt_s - dsm) + (size_t)max(n_rows + 1, n_st) * 16 <= (size_t)P.smem_bytes) {
+                xtab = xt_s;
+                ktab = stage = kt_s;
+                KChunk* cs = reinterpret_cast<KChunk*>(xt_s + n_x + 1);
                 for (int t = tid; t <= n_x; t += blockDim.x) xtab[t] = xg[t];
                 for (int t = tid; t < n_ch; t += blockDim.x) cs[t] = chunks[t];
                 chk = cs;
             } else {   // slower, but any number of rows
                 tab_smem = false;
+                stage = reinterpret_cast<int4*>(dsm + off);
                 xtab = xg;
                 ktab = reinterpret_cast<int4*>(slot + P.off_ktab);
                 acc = cpart + 4 * kMaxLocalProjAtoms;
@@ -891,7 +913,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 cf[t] = P.proj_fxc[4LL * SN[0].la_id[t >> 2] + (t & 3)] / P.scale * 0x1p-62;
             }
             __syncthreads();
-            if (tid == 0) xtab[0] = ktab[0] = make_int4(0, 0, 0, 0);
+            if (tid == 0) xtab[0] = make_int4(0, 0, 0, 0);
         }
         const SlabArgs SA{U, Vp, Wp, Rec, m0, m1, npx, npc, n_items, pitch, pp,
                           make_fastdiv((uint32_t)npc), div_px};
@@ -904,13 +926,13 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         k_sync();
         int bad = 0;
         for (int r = 0; r < C; ++r) bad = max(bad, (int)S.mbox[r][4]);
-        // u_1 = e_j / 4, pushed to every CTA whose slab or halo holds the plane
+        // u_1 = e_j / 8, pushed to every CTA whose slab or halo holds the plane
         if (tid == 0) {
             const int b = src_col / m0, a = src_col - b * m0;
             if (src_z >= z0 - Q && src_z < z0 + depth + Q)
-                U[(src_z - z0 + Q) * pp + b * pitch + a] = split31(1LL << 60);
-            S.s0 = 0x1p-4;
-            S.inv0 = 0x1p4;
+                U[(src_z - z0 + Q) * pp + b * pitch + a] = split31(1LL << 59);
+            S.s0 = 0x1p-6;
+            S.inv0 = 0x1p6;
             S.cg = make_int2(0, 0);
             S.stop = 0;
             S.a_hat = 0.0;
@@ -922,7 +944,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         if (scalar_warp && rank == 0 && P.K == 0) {
             for (int k = lane; k < P.P; k += 32, ++np) {
                 const double2 z = P.z[k];
-                ps[np] = PoleState{(z.x - P.shift) / P.scale, z.y / P.scale, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0, 1.0, 0, 0, 4.0, 0.0,
+                ps[np] = PoleState{(z.x - P.shift) / P.scale, z.y / P.scale, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0, 1.0, 0, 0, 8.0, 0.0,
                                    0.0, 0.0};
             }
         }
@@ -988,14 +1010,15 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                     long long s = 0;
                     for (int r = 0; r < C; ++r)
                         s += __ldcg(reinterpret_cast<const long long*>(slot0 + (size_t)r * P.cta_bytes + P.off_cpart) + t);
-                    cl[t] = to_limbs((double)s * cf[t]);
+                    cl[t] = tab_limbs(to_limbs((double)s * cf[t]));
                 }
                 __syncthreads();
 #pragma unroll 4
                 for (int t = tid; t < n_rows; t += blockDim.x) ktab[t + 1] = row_factors(rows + t, cl);
+                if (tid == 0) ktab[0] = make_int4(0, 0, 0, 0);
                 __syncthreads();
             }
-            long long hh1 = 0, l1 = 0, hh2 = 0, l2 = 0;
+            Dots dots;
             if (scalar_warp) {
                 // pole recurrences of the step before, while the others compute
                 if (rank == 0 && P.K == 0) {
@@ -1011,30 +1034,22 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 const int2 g = make_int2(-S.cg.x, -S.cg.y);
                 const int4* up = Up + (size_t)((it - 1 + ring) % ring) * n_items;
                 // (the compiler sees that these tables are in shared memory)
-                if (!kNl || tab_smem) slab_apply<Q, kNl>(P, SA, stab + n_x + 1, stab, up, nwp, g, hh1, l1, hh2, l2);
-                else slab_apply<Q, kNl>(P, SA, ktab, xtab, up, nwp, g, hh1, l1, hh2, l2);
+                if (!kNl || tab_smem) slab_apply<Q, kNl>(P, SA, kt_s, xt_s, up, nwp, g, dots);
+                else slab_apply<Q, kNl>(P, SA, ktab, xtab, up, nwp, g, dots);
             }
             // ---- u.w and w.w over the cluster ------------------------------
             if (!scalar_warp) {
-                hh1 = warp_sum_i(hh1);
-                l1 = warp_sum_i(l1);
-                hh2 = warp_sum_i(hh2);
-                l2 = warp_sum_i(l2);
-                if (lane == 0) {
-                    S.part[warp][0] = hh1;
-                    S.part[warp][1] = l1;
-                    S.part[warp][2] = hh2;
-                    S.part[warp][3] = l2;
-                }
+                const long long s = warp_sum4(dots.hh1, dots.l1(), dots.hh2, dots.l2(), lane);
+                if (lane < 4) S.part[warp][lane] = s;
             }
             __syncthreads();
             if (scalar_warp) {
-                long long t[5];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) t[k] = warp_sum_i(lane < nwp ? S.part[lane][k] : 0LL);
-                t[4] = rank == 0 ? S.stop : 0;
-                if (lane < C)
-                    for (int k = 0; k < 5; ++k) k_st_remote(k_map(smem_addr(&S.mbox[rank][k]), lane), t[k]);
+                const bool on = lane < nwp;
+                const long long s = warp_sum4(on ? S.part[lane][0] : 0LL, on ? S.part[lane][1] : 0LL,
+                                              on ? S.part[lane][2] : 0LL, on ? S.part[lane][3] : 0LL, lane);
+                // lanes 4 r + k: value k to rank r (C <= 8); warp_sum4 leaves value lane mod 4 in every lane
+                if ((lane >> 2) < C) k_st_remote(k_map(smem_addr(&S.mbox[rank][lane & 3]), lane >> 2), s);
+                if (rank == 0 && lane < C) k_st_remote(k_map(smem_addr(&S.mbox[0][4]), lane), (long long)S.stop);
             }
             k_sync();
             ++it;
@@ -1066,28 +1081,38 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 } else if (it >= P.maxit && !st) {
                     st = 1;
                 }
-                // ||u_new||^2 = n2 4^e in [1/16, 1/4)
+                // ||u_new||^2 = n2 4^e in [1/64, 1/16)
                 // (n2 >= 2^-116 here, or the node stops)
                 const int ex = max(((__double2hiint(n2) >> 20) & 0x7ff) - 1022, -120);
-                const int e = min(40, (-2 - ex) >> 1);
-                const double p2 = __hiloint2double((1023 + e) << 20, 0);   // 2^e
-                const double s0n = n2 * p2 * p2;
-                const double gn = n2 * p2 * S.inv0;
-                const int2 ca = to_limbs(al), cg = to_limbs(gn);
+                const int e = min(40, (-4 - ex) >> 1);
+                const int2 ca = to_limbs(al);
                 __syncwarp();
                 if (lane == 0) {
-                    S.cg_used = S.cg;
                     S.ca = ca;
-                    S.cg = cg;
                     S.e = e;
                     S.stop = st;
+                }
+                __syncthreads();
+                // the rest while the others form u_new
+                const double p2 = __hiloint2double((1023 + e) << 20, 0);   // 2^e
+                const double s0n = n2 * p2 * p2;
+                const int2 cg = to_limbs(n2 * p2 * S.inv0);
+                const double inv = 1.0 / s0n;
+                __syncwarp();
+                if (lane == 0) {
                     S.a_hat = al;
                     S.b2_hat = b2;
                     S.e_hat = e;
-                    S.s0 = s0n;
+                    if (!st) {
+                        S.cg = cg;
+                        S.s0 = s0n;
+                        S.inv0 = inv;
+                    }
                 }
+                __syncwarp();
+            } else {
+                __syncthreads();
             }
-            __syncthreads();
             stop = S.stop;
             if (P.vec && (stop || it % kKryVec == 0)) {
                 // apply the vectors kept to the solutions
@@ -1125,10 +1150,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 k_sync();   // from here the coefficients may be written again
             }
             if (stop) break;
-            if (scalar_warp) {
-                if (lane == 0) S.inv0 = 1.0 / S.s0;
-            } else {
+            if (!scalar_warp) {
                 const int2 al = S.ca;
+                const f32x2 alf = lo_hi(al.x, al.y);
                 const int e = S.e;
                 const uint32_t ubase = smem_addr(U);
                 // two pairs at a time: their loads are in flight together
@@ -1147,11 +1171,11 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                         const int idx = pb * pitch + 2 * (pc - pb * npx);
                         int4* up = reinterpret_cast<int4*>(U + (d + Q) * pp + idx);
                         const int4 u = *up;
-                        const int ax = opaque(al.x), ay = opaque(al.y);
-                        long long h0 = 0, h1 = 0, g0 = kHalf, g1 = kHalf;
-                        mac(h0, g0, u.x, u.y, ax, ay);
-                        mac(h1, g1, u.z, u.w, ax, ay);
-                        const long long t0 = w[j].x - fold(h0, g0), t1 = w[j].y - fold(h1, g1);
+                        const int ax = opaque(al.x);
+                        Acc a0, a1;
+                        a0.mac(u.x, hi_lo(u.x, u.y), ax, alf);
+                        a1.mac(u.z, hi_lo(u.z, u.w), ax, alf);
+                        const long long t0 = w[j].x - a0.fold(), t1 = w[j].y - a1.fold();
                         const int2 a = split31(e >= 0 ? t0 << e : t0 >> -e), b = split31(e >= 0 ? t1 << e : t1 >> -e);
                         const int4 nu = make_int4(a.x, a.y, b.x, b.y);
                         Up[(size_t)((it - 1) % ring) * n_items + item] = u;
@@ -1174,7 +1198,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         if (P.check && !bad) {
             double* c = reinterpret_cast<double*>(acc);   // free once the steps are done
             double* part = reinterpret_cast<double*>(cpart);
-            double s2 = check_step<Q, kNl>(P, SA, lo, z0, SN[0], c, Up + (size_t)((it - 2 + ring) % ring) * n_items, S.cg_used, [&]() {
+            double s2 = check_step<Q, kNl>(P, SA, lo, z0, SN[0], c, Up + (size_t)((it - 2 + ring) % ring) * n_items, S.cg, [&]() {
                 __syncthreads();
                 for (int t = tid; t < n_loc4; t += blockDim.x) part[t] = c[t];
                 k_sync();
@@ -1291,7 +1315,8 @@ __global__ void k_proj_fixed(long long n_atoms, const int* __restrict__ len, con
             const bool in = u < len[3 * a + warp];
             const double g = in ? gtab[base + u] : 0.0, dg = in ? dtab[base + u] * g : 0.0;
             const int2 x = to_limbs(g * ig), y = to_limbs(dg * id);
-            fx[base + u] = make_int4(x.x, x.y, y.x, y.y);
+            const int2 a_ = tab_limbs(x), b_ = tab_limbs(y);
+            fx[base + u] = make_int4(a_.x, a_.y, b_.x, b_.y);
         }
     }
     __syncthreads();
