@@ -193,10 +193,19 @@ __global__ void __launch_bounds__(1024) k_lanczos(const __grid_constant__ SolveP
     }
 }
 
+// A column of a [K][32] array in shared memory: entry k of this thread's node.
+struct Column {
+    double* p;
+    __device__ __forceinline__ double& operator[](int k) const { return p[32 * k]; }
+};
+
 // Eigenvalues and first-row eigenvector components of the n x n Jacobi
 // matrix (d, e) in place; returns false if some eigenvalue did not converge
-// within 30 n steps.
-__device__ bool jacobi_eig_first_row(int n, double* d, double* e, double* z) {
+// within 30 n steps.  A serial chain of dependent FP64 operations, so what
+// counts is its length: the rotation takes one reciprocal square root (a
+// hypot and two divisions made the 256 rules of K = 40 take 5 ms, a fifth of
+// the whole call).
+__device__ bool jacobi_eig_first_row(int n, Column d, Column e, Column z) {
     for (int i = 0; i < n; ++i) z[i] = (i == 0) ? 1.0 : 0.0;
     int hi = n - 1;
     int steps = 0;
@@ -216,38 +225,46 @@ __device__ bool jacobi_eig_first_row(int n, double* d, double* e, double* z) {
         const double mu = d[hi] - b2 / (delta + copysign(sqrt(delta * delta + b2), delta));
         // bulge chase: rotation k acts on rows / columns k, k+1; its first
         // one is fixed by the first column of T - mu I
-        double x = d[lo] - mu, y = e[lo];
+        double ak = d[lo], bk = e[lo], zk = z[lo];
+        double x = ak - mu, y = bk;
         for (int k = lo; k < hi; ++k) {
-            const double r = hypot(x, y);
-            double c = 1.0, s = 0.0;
-            if (r > 0.0) {
-                c = x / r;
-                s = y / r;
+            const double ak1 = d[k + 1], zk1 = z[k + 1], bk1 = k + 1 < hi ? e[k + 1] : 0.0;
+            const double r2 = x * x + y * y;
+            double c = 1.0, s = 0.0, r = 0.0;
+            if (r2 > 1e-280) {
+                const double inv = rsqrt(r2);
+                c = x * inv;
+                s = y * inv;
+                r = r2 * inv;
+            } else {            // the squares underflow
+                r = hypot(x, y);
+                if (r > 0.0) {
+                    c = x / r;
+                    s = y / r;
+                }
             }
             if (k > lo) e[k - 1] = r;
-            const double ak = d[k], ak1 = d[k + 1], bk = e[k];
             d[k] = c * c * ak + 2.0 * c * s * bk + s * s * ak1;
-            d[k + 1] = s * s * ak - 2.0 * c * s * bk + c * c * ak1;
-            e[k] = c * s * (ak1 - ak) + (c * c - s * s) * bk;
-            if (k + 1 < hi) {
-                const double bk1 = e[k + 1];
-                y = s * bk1;          // bulge at (k+2, k)
-                e[k + 1] = c * bk1;
-                x = e[k];
-            }
-            const double zk = z[k], zk1 = z[k + 1];
+            x = c * s * (ak1 - ak) + (c * c - s * s) * bk;   // the new e[k]
+            ak = s * s * ak - 2.0 * c * s * bk + c * c * ak1;
+            y = s * bk1;        // bulge at (k+2, k)
+            bk = c * bk1;
             z[k] = c * zk + s * zk1;
-            z[k + 1] = c * zk1 - s * zk;
+            zk = c * zk1 - s * zk;
         }
+        d[hi] = ak;
+        e[hi - 1] = x;
+        z[hi] = zk;
     }
     return true;
 }
 
-__global__ void k_gauss_rules(int n_nodes, const LanczosParams L, double* __restrict__ lambda,
-                              double* __restrict__ weight) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(32) k_gauss_rules(int n_nodes, const LanczosParams L, double* __restrict__ lambda,
+                                                    double* __restrict__ weight) {
+    extern __shared__ double cols[];
+    const int j = blockIdx.x * 32 + threadIdx.x;
     if (j >= n_nodes) return;
-    double d[kMaxLanczosK], e[kMaxLanczosK], z[kMaxLanczosK];
+    const Column d{cols + threadIdx.x}, e{d.p + 32 * L.K}, z{e.p + 32 * L.K};
     const long long base = (long long)j * L.K;
     const int n = L.k_used[j];
     if (n <= 0) {
@@ -410,7 +427,10 @@ cudaError_t launch_lanczos(const SolveParams& P, const LanczosParams& L, int pre
 cudaError_t launch_gauss_rules(int n_nodes, const LanczosParams& L, double* lambda, double* weight,
                                cudaStream_t stream) {
     if (n_nodes <= 0) return cudaSuccess;
-    k_gauss_rules<<<(n_nodes + 63) / 64, 64, 0, stream>>>(n_nodes, L, lambda, weight);
+    const size_t smem = (size_t)3 * 32 * L.K * sizeof(double);   // 96 KiB at K = 128
+    const cudaError_t e = cudaFuncSetAttribute(k_gauss_rules, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_gauss_rules<<<(n_nodes + 31) / 32, 32, smem, stream>>>(n_nodes, L, lambda, weight);
     return cudaGetLastError();
 }
 
