@@ -91,28 +91,210 @@ struct CellArgs {
     const int* atoms;
 };
 
-__global__ void k_local_potential(GridGeo g, CellArgs cl, const double* __restrict__ xyz,
-                                  const double* __restrict__ depth, const double* __restrict__ sigma,
-                                  double cutoff_sigmas, const double* __restrict__ v_ext,
-                                  double* __restrict__ V, float* __restrict__ V32, long long N) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ix = (int)(i % g.n[0]);
-        const int iy = (int)((i / g.n[0]) % g.n[1]);
-        const int iz = (int)(i / ((long long)g.n[0] * g.n[1]));
-        const double px = ix * g.h[0], py = iy * g.h[1], pz = iz * g.h[2];
-        double v = v_ext ? v_ext[i] : 0.0;
-        for_each_near_atom(g, cl.nc, cl.cell, cl.start, cl.atoms, ix, iy, iz, [&](int a) {
-            const double dx = min_image(px - xyz[3 * a + 0], g.L[0], g.periodic[0]);
-            const double dy = min_image(py - xyz[3 * a + 1], g.L[1], g.periodic[1]);
-            const double dz = min_image(pz - xyz[3 * a + 2], g.L[2], g.periodic[2]);
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            const double s = sigma[a];
-            const double rc = cutoff_sigmas * s;
-            if (r2 <= rc * rc) v -= depth[a] * exp(-r2 / (2.0 * s * s));
-        });
-        V[i] = v;
-        V32[i] = (float)v;
+// Wells summed over a tile of 32 x 8 x 8 points per block.  The Gaussian is a
+// product of three 1-D factors, so each atom near the tile needs only 48
+// exponentials and squared displacements, kept in shared memory; a point and
+// atom then cost an addition, a comparison and a multiply-add in FP64 (the
+// scarce pipe here: 1.7 a clock and SM), and columns outside the sphere are
+// skipped.  One exponential and three minimum-image divisions per point and
+// atom took 21 ms on the 96 x 96 x 160 grid with 1,024 atoms.
+constexpr int kTx = 32, kTy = 8, kTz = 8;      // tile
+constexpr int kTab = kTx + kTy + kTz;
+constexpr int kAtomBatch = 16;                 // atoms tabulated at a time
+constexpr int kNear = 512;                     // atoms of the list in shared memory
+
+// Lower bound of the squared distance from X to the points lo..hi (grid
+// indices) on one axis.
+__device__ __forceinline__ double axis_gap(double X, double lo, double hi, double L, int periodic) {
+    const double c = 0.5 * (lo + hi), r = 0.5 * (hi - lo);
+    const double d = fabs(min_image(X - c, L, periodic)) - r;
+    return d > 0.0 ? d * d : 0.0;
+}
+
+__global__ void __launch_bounds__(kTx* kTy) k_local_potential(
+    GridGeo g, CellArgs cl, const double* __restrict__ xyz, const double* __restrict__ depth,
+    const double* __restrict__ sigma, double cutoff_sigmas, double reach, const double* __restrict__ v_ext,
+    double* __restrict__ V, float* __restrict__ V32, int tiles_x, int tiles_y, long long n_tiles) {
+    __shared__ int near_id[kNear];
+    __shared__ double2 tab[kAtomBatch][kTab];   // squared displacement, Gaussian factor
+    __shared__ double2 par[kAtomBatch];         // depth, squared cutoff
+    __shared__ int warp_n[kTx * kTy / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kTx * kTy / 32;
+    const int tx = tid % kTx, ty = tid / kTx;
+    for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        const int o[3] = {(int)(tile % tiles_x) * kTx, (int)((tile / tiles_x) % tiles_y) * kTy,
+                          (int)(tile / ((long long)tiles_x * tiles_y)) * kTz};
+        const int ext[3] = {kTx, kTy, kTz};
+        double lo[3], hi[3];
+        int c0[3], nc[3];   // first cell and number of cells that can hold atoms in reach
+        for (int d = 0; d < 3; ++d) {
+            lo[d] = o[d] * g.h[d];
+            hi[d] = (min(o[d] + ext[d], g.n[d]) - 1) * g.h[d];
+            int a = (int)floor((lo[d] - reach) / cl.cell[d]), b = (int)floor((hi[d] + reach) / cl.cell[d]);
+            if (g.periodic[d]) {
+                if (b - a + 1 >= cl.nc[d]) a = 0, b = cl.nc[d] - 1;
+            } else {
+                a = min(max(a, 0), cl.nc[d] - 1);
+                b = min(max(b, 0), cl.nc[d] - 1);
+            }
+            c0[d] = a;
+            nc[d] = b - a + 1;
+        }
+        double acc[kTz];
+#pragma unroll
+        for (int z = 0; z < kTz; ++z) acc[z] = 0.0;
+        int n_near = 0;
+        // the listed atoms, a batch at a time
+        auto sum_near = [&]() {
+            for (int a0 = 0; a0 < n_near; a0 += kAtomBatch) {
+                const int na = min(kAtomBatch, n_near - a0);
+                __syncthreads();
+                for (int t = tid; t < na * kTab; t += blockDim.x) {
+                    const int k = t / kTab, i = t - k * kTab;
+                    const int d = i < kTx ? 0 : (i < kTx + kTy ? 1 : 2);
+                    const int idx = o[d] + i - (d == 0 ? 0 : (d == 1 ? kTx : kTx + kTy));
+                    const int at = near_id[a0 + k];
+                    const double s = sigma[at];
+                    const double dd = min_image(idx * g.h[d] - xyz[3 * at + d], g.L[d], g.periodic[d]);
+                    tab[k][i] = make_double2(dd * dd, exp(-dd * dd / (2.0 * s * s)));
+                    if (i == 0) {
+                        const double rc = cutoff_sigmas * s;
+                        par[k] = make_double2(depth[at], rc * rc);
+                    }
+                }
+                __syncthreads();
+                for (int k = 0; k < na; ++k) {
+                    const double2 p = par[k], x = tab[k][tx], y = tab[k][kTx + ty];
+                    const double dxy = x.x + y.x;
+                    if (dxy > p.y) continue;
+                    const double gxy = p.x * x.y * y.y;
+#pragma unroll
+                    for (int z = 0; z < kTz; ++z) {
+                        const double2 w = tab[k][kTx + kTy + z];
+                        if (dxy + w.x <= p.y) acc[z] = fma(gxy, w.y, acc[z]);
+                    }
+                }
+            }
+            __syncthreads();
+            n_near = 0;
+        };
+        // cells in order, one per warp at a time; the list order is fixed, so
+        // that a potential comes out the same every time
+        const int n_cells = nc[0] * nc[1] * nc[2];
+        for (int cb = 0; cb < n_cells; cb += nw) {
+            int e = lane, end = 0;
+            if (cb + warp < n_cells) {
+                const int c = cb + warp;
+                int k[3] = {c0[0] + c % nc[0], c0[1] + (c / nc[0]) % nc[1], c0[2] + c / (nc[0] * nc[1])};
+                for (int d = 0; d < 3; ++d) k[d] = ((k[d] % cl.nc[d]) + cl.nc[d]) % cl.nc[d];
+                const int cell = k[0] + cl.nc[0] * (k[1] + cl.nc[1] * k[2]);
+                e = cl.start[cell] + lane;
+                end = cl.start[cell + 1];
+            }
+            while (__syncthreads_or(e - lane < end)) {
+                bool in = false;
+                int at = 0;
+                if (e < end) {
+                    at = cl.atoms[e];
+                    const double rc = cutoff_sigmas * sigma[at];
+                    double r2 = 0.0;
+                    for (int d = 0; d < 3; ++d) r2 += axis_gap(xyz[3 * at + d], lo[d], hi[d], g.L[d], g.periodic[d]);
+                    in = r2 <= rc * rc * (1.0 + 1e-9);
+                }
+                e += 32;
+                const unsigned m = __ballot_sync(0xffffffffu, in);
+                if (lane == 0) warp_n[warp] = __popc(m);
+                __syncthreads();
+                int before = n_near, total = n_near;
+                for (int w = 0; w < nw; ++w) {
+                    if (w < warp) before += warp_n[w];
+                    total += warp_n[w];
+                }
+                if (in) near_id[before + __popc(m & ((1u << lane) - 1u))] = at;
+                n_near = total;
+                __syncthreads();
+                if (n_near > kNear - kTx * kTy) sum_near();
+            }
+        }
+        sum_near();
+        const int ix = o[0] + tx, iy = o[1] + ty;
+        if (ix < g.n[0] && iy < g.n[1]) {
+#pragma unroll
+            for (int z = 0; z < kTz; ++z) {
+                if (o[2] + z >= g.n[2]) break;
+                const long long i = ix + (long long)g.n[0] * (iy + (long long)g.n[1] * (o[2] + z));
+                const double v = (v_ext ? v_ext[i] : 0.0) - acc[z];
+                V[i] = v;
+                V32[i] = (float)v;
+            }
+        }
+    }
+}
+
+// Exclusive prefix sum of the list lengths: sums of 2,048 points, the sums'
+// prefix in one block, then the points.
+constexpr int kScan = 2048;
+
+__device__ __forceinline__ long long block_exclusive(long long v, long long* tmp, long long& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    long long x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    __syncthreads();
+    if (lane == 31) tmp[warp] = x;
+    __syncthreads();
+    long long before = 0;
+    total = 0;
+    for (int w = 0; w < nw; ++w) {
+        if (w < warp) before += tmp[w];
+        total += tmp[w];
+    }
+    return before + x - v;
+}
+
+// head[0] = entries in all, head[1] = the longest list
+__global__ void __launch_bounds__(256) k_scan_sums(const int* __restrict__ cnt, long long N, long long* sums,
+                                                   long long* head) {
+    __shared__ long long tmp[8];
+    const long long base = (long long)blockIdx.x * kScan;
+    long long s = 0;
+    int mx = 0;
+    for (int i = threadIdx.x; i < kScan && base + i < N; i += blockDim.x) {
+        s += cnt[base + i];
+        mx = max(mx, cnt[base + i]);
+    }
+    long long total;
+    block_exclusive(s, tmp, total);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(head + 1, (long long)mx);
+    if (threadIdx.x == 0) sums[blockIdx.x] = total;
+}
+__global__ void __launch_bounds__(1024) k_scan_blocks(long long* sums, long long n, long long* head) {
+    __shared__ long long tmp[32];
+    long long run = 0;
+    for (long long b = 0; b < n; b += blockDim.x) {
+        const long long i = b + threadIdx.x;
+        long long total;
+        const long long x = block_exclusive(i < n ? sums[i] : 0LL, tmp, total);
+        if (i < n) sums[i] = run + x;
+        run += total;
+    }
+    if (threadIdx.x == 0) head[0] = run;
+}
+__global__ void __launch_bounds__(256) k_scan_points(const int* __restrict__ cnt, long long N,
+                                                     const long long* __restrict__ sums, int* __restrict__ ptr) {
+    __shared__ long long tmp[8];
+    const long long base = (long long)blockIdx.x * kScan;
+    long long run = sums[blockIdx.x];
+    for (int b = 0; b < kScan; b += blockDim.x) {
+        const long long i = base + b + threadIdx.x;
+        long long total;
+        const long long x = block_exclusive(i < N ? cnt[i] : 0, tmp, total);
+        if (i <= N) ptr[i] = (int)(run + x);
+        run += total;
     }
 }
 
@@ -487,6 +669,7 @@ md_status build_hamiltonian_device(Ham& H, const md_atoms* atoms, const md_pot_p
     double* d_vext = nullptr;
     int* d_overflow = nullptr;
     int* d_count = nullptr;
+    long long* d_sums = nullptr;
     double max_sigma = 0.0;
     GridGeo g = geo_of(H);
     const int threads = 256;
@@ -524,8 +707,13 @@ md_status build_hamiltonian_device(Ham& H, const md_atoms* atoms, const md_pot_p
     }
     ca.start = d_cstart;
     ca.atoms = d_cids;
-    k_local_potential<<<blocks, threads, 0, stream>>>(g, ca, H.atom_xyz, H.atom_depth, H.atom_sigma,
-                                                     H.cutoff_sigmas, d_vext, H.V, H.V32, N);
+    {
+        const int tx = (H.n[0] + kTx - 1) / kTx, ty = (H.n[1] + kTy - 1) / kTy;
+        const long long tiles = (long long)tx * ty * ((H.n[2] + kTz - 1) / kTz);
+        k_local_potential<<<(unsigned)std::min<long long>(tiles, 152LL * 64), kTx * kTy, 0, stream>>>(
+            g, ca, H.atom_xyz, H.atom_depth, H.atom_sigma, H.cutoff_sigmas, H.cutoff_sigmas * max_sigma, d_vext, H.V,
+            H.V32, tx, ty, tiles);
+    }
     MD_CUDA_TRY(cudaGetLastError());
 
     if (H.nonlocal && H.n_atoms > 0) {
@@ -579,9 +767,17 @@ md_status build_hamiltonian_device(Ham& H, const md_atoms* atoms, const md_pot_p
                                                             nullptr, nullptr, nullptr, d_overflow);
         MD_CUDA_TRY(cudaGetLastError());
         {
-            std::vector<int> cnt(N + 1, 0);
+            const long long nb = N / kScan + 1;   // the last block also writes entry N
+            long long head[2] = {0, 0};
             int ovf[2] = {0, 0};
-            MD_CUDA_TRY(cudaMemcpyAsync(cnt.data(), d_count, N * sizeof(int), cudaMemcpyDeviceToHost, stream));
+            MD_CUDA_TRY(cudaMalloc(&d_sums, (nb + 2) * sizeof(long long)));
+            MD_CUDA_TRY(cudaMalloc(&H.pl_ptr, (N + 1) * sizeof(int)));
+            MD_CUDA_TRY(cudaMemsetAsync(d_sums, 0, 2 * sizeof(long long), stream));
+            k_scan_sums<<<(unsigned)nb, 256, 0, stream>>>(d_count, N, d_sums + 2, d_sums);
+            k_scan_blocks<<<1, 1024, 0, stream>>>(d_sums + 2, nb, d_sums);
+            k_scan_points<<<(unsigned)nb, 256, 0, stream>>>(d_count, N, d_sums + 2, H.pl_ptr);
+            MD_CUDA_TRY(cudaGetLastError());
+            MD_CUDA_TRY(cudaMemcpyAsync(head, d_sums, sizeof(head), cudaMemcpyDeviceToHost, stream));
             MD_CUDA_TRY(cudaMemcpyAsync(ovf, d_overflow, sizeof(ovf), cudaMemcpyDeviceToHost, stream));
             MD_CUDA_TRY(cudaStreamSynchronize(stream));
             H.proj_fx_ok = ovf[1] == 0;
@@ -589,24 +785,16 @@ md_status build_hamiltonian_device(Ham& H, const md_atoms* atoms, const md_pot_p
                 st = set_error(MD_ERR_INVALID, "md_build_hamiltonian: more than 16 projector atoms at one grid point");
                 goto fail;
             }
-            long long run = 0;
-            for (long long i = 0; i < N; ++i) {
-                const long long c = cnt[i];
-                H.pl_max = std::max(H.pl_max, cnt[i]);
-                if (run > 2147483647LL - 16) {
-                    st = set_error(MD_ERR_INVALID, "md_build_hamiltonian: too many projector entries (2^31)");
-                    goto fail;
-                }
-                cnt[i] = (int)run;
-                run += c;
+            const long long run = head[0];
+            if (run > 2147483647LL - 16) {
+                st = set_error(MD_ERR_INVALID, "md_build_hamiltonian: too many projector entries (2^31)");
+                goto fail;
             }
-            cnt[N] = (int)run;
+            H.pl_max = (int)head[1];
             H.pl_nnz = run;
-            MD_CUDA_TRY(cudaMalloc(&H.pl_ptr, (N + 1) * sizeof(int)));
             MD_CUDA_TRY(cudaMalloc(&H.pl_atom, std::max<long long>(run, 1) * sizeof(int)));
             MD_CUDA_TRY(cudaMalloc(&H.pl_val32, std::max<long long>(run, 1) * sizeof(float4)));
             MD_CUDA_TRY(cudaMalloc(&H.pl_val64, std::max<long long>(run, 1) * 2 * sizeof(double2)));
-            MD_CUDA_TRY(cudaMemcpy(H.pl_ptr, cnt.data(), (N + 1) * sizeof(int), cudaMemcpyHostToDevice));
         }
         k_proj_lists<true><<<blocks, threads, 0, stream>>>(g, ca, H.proj_i0, H.proj_len, H.proj_rows,
                                                            H.proj_d, H.proj_g, H.proj_C, N, H.pl_ptr,
@@ -627,6 +815,7 @@ fail:
     cudaFree(d_vext);
     cudaFree(d_overflow);
     cudaFree(d_count);
+    cudaFree(d_sums);
     return st;
 }
 
