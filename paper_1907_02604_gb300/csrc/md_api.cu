@@ -353,10 +353,12 @@ KryShape kry_shape(const Ham& H, int m0, int m1, int m2, int c, int dev) {
     s.per_sm = std::max(1, std::min({(int)(232448 / (s.smem + kry_static_smem_bytes(nl) + 1024)), 2048 / s.block,
                                      24 / (s.block / 32)}));
     s.clusters = kry_clusters_alone(c) * s.per_sm;
-    // a step, measured in cycles: 8 a warp's 32 pairs and warp in flight (11 with
-    // projectors), 3,000 a plane for the projections, the exchanges
-    s.time = s.per_sm * best * (nl ? (s.spill ? 22.0 : 11.0) : 8.0) +
-             (nl ? 18000.0 + s.per_sm * 3000.0 * s.depth * (m0 * m1 / 1089.0) : 8000.0);
+    // a step in cycles, measured on 33^3 and 41^3 regions: the slab's passes
+    // (190 a round and warp in flight with projectors, 236 with their tables in
+    // device memory, 138 without), 2,600 a 33 x 33 plane for the projections,
+    // and the exchanges
+    s.time = s.per_sm * best * (nl ? (s.spill ? 236.0 : 190.0) : 138.0) +
+             (nl ? 17000.0 + s.per_sm * 2600.0 * s.depth * (m0 * m1 / 1089.0) : 7500.0);
     s.csz = c;
     return s;
 }
@@ -396,24 +398,40 @@ bool kry_classes(const Ham& H, const Regions& R, std::vector<int>& order, std::v
         }
         if (cand[k].empty()) return false;
     }
-    // Krylov steps grow about linearly with the region's extent.  One class:
-    // the shape with the shortest makespan.  Several share the device: each
-    // takes the shape with the least SM time, then those whose nodes alone
-    // would outlast the rest move to more CTAs a node.
+    // One class: the shape with the shortest makespan, the nodes left over
+    // after its last full wave with a shape of their own (96 bulk nodes on 36
+    // clusters of four CTAs: two waves and 24 nodes on clusters of six)
     shapes.assign(nc, KryShape{});
     if (nc == 1) {
         double best = 0.0;
+        KryShape tail;
+        int full = nn;
         for (const KryShape& s : cand[0]) {
-            const double t = std::ceil((double)nn / s.clusters) * s.time;
-            const double alone = nn <= s.clusters / s.per_sm ? s.time / s.per_sm : t;
-            const double v = std::min(t, std::max(alone, 0.0));
-            if (shapes[0].csz == 0 || v < 0.98 * best) {
-                best = v;
+            const int waves = nn / s.clusters, rest = nn - waves * s.clusters;
+            auto offer = [&](double t, int n1, const KryShape& s2) {
+                if (shapes[0].csz != 0 && t >= 0.98 * best) return;
+                best = t;
                 shapes[0] = s;
-            }
+                full = n1;
+                tail = s2;
+            };
+            // (a wave that leaves SMs idle still takes a whole step's time, at most one CTA an SM)
+            const double last = rest <= s.clusters / s.per_sm ? s.time / s.per_sm : s.time;
+            offer(waves * s.time + (rest ? last : 0.0), nn, s);
+            if (waves > 0 && rest > 0)
+                for (const KryShape& s2 : cand[0])
+                    if (s2.csz > s.csz && rest <= s2.clusters) offer(waves * s.time + s2.time, nn - rest, s2);
+        }
+        if (full < nn) {
+            first = {0, full, nn};
+            shapes.push_back(tail);
+            dims.push_back(dims[0]);
         }
         return true;
     }
+    // Several share the device (Krylov steps grow about linearly with the
+    // region's extent): each takes the shape with the least SM time, then
+    // those whose nodes alone would outlast the rest move to more CTAs a node.
     double total = 0.0;
     auto sm_time = [&](int k, const KryShape& s) {
         return (double)(first[k + 1] - first[k]) * s.time * dims[k].dims[2] / s.clusters;

@@ -206,7 +206,7 @@ struct KShared {
 struct VecHead {      // one pole's update of its solution vector
     double sw, sv;    // powers of two the coefficients were divided by
     double2 om, nu;
-    int act, first;
+    int act, first, last;   // last: the solution is complete, no further direction
 };
 struct KSharedVec {
     int4 co[4 * kKryVec];         // coefficients of the pole in hand
@@ -735,6 +735,7 @@ __device__ void vec_coefs(const VecHist* hist, int n, int s0, PoleState& s, int 
             head->nu = make_double2(-(s.mr * v.x - s.mi * v.y), -(s.mr * v.y + s.mi * v.x));
             head->act = s.frz == 0 || s.frz > s0;
             head->first = s0 == 0;
+            head->last = s.frz != 0;
         }
     }
     const double2 m = hist[(size_t)(n - 1) * kKryMaxPoles + pole].m;
@@ -745,7 +746,7 @@ __device__ void vec_coefs(const VecHist* hist, int n, int s0, PoleState& s, int 
 // x and p of one pole over the slab: fixed-point sums over the kept vectors
 // (the mixed terms in float, 2^-55 of the sum), joined in FP64.  A pair's
 // first point lies at X[xoff(item)], the second beside it.
-template <class F>
+template <bool kLast, class F>
 __device__ __forceinline__ void vec_update(const SlabArgs& A, int n, const int4* co, const VecHead& h, const int4* Ub,
                                            double2* X, double2* Pv, F&& xoff) {
     const double sx = h.sw * 0x1p-62, sp = h.sv * 0x1p-62;
@@ -759,7 +760,7 @@ __device__ __forceinline__ void vec_update(const SlabArgs& A, int n, const int4*
             up += A.n_items;
             const float a0 = (float)u.x, b0 = (float)u.y, a1 = (float)u.z, b1 = (float)u.w;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
+            for (int k = 0; k < (kLast ? 2 : 4); ++k) {
                 const int4 c = co[4 * j + k];
                 const float ch = __int_as_float(c.y), cl = __int_as_float(c.z);
                 madw(hh[2 * k], u.x, c.x);
@@ -786,7 +787,7 @@ __device__ __forceinline__ void vec_update(const SlabArgs& A, int n, const int4*
                 pv.y += h.nu.x * po.y + h.nu.y * po.x;
             }
             x[i] = xv;
-            p[i] = pv;
+            if (!kLast) p[i] = pv;
         }
     }
 }
@@ -1144,7 +1145,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                     __syncthreads();
                     double2* x = P.ckpt ? P.ckpt + P.ckpt_off[(long long)node * P.P + pole]
                                         : Xs + (size_t)pole * 2 * n_items;
-                    vec_update(SA, n, SV.co, SV.head, Up, x, Ps + (size_t)pole * 2 * n_items, vec_index);
+                    double2* pv = Ps + (size_t)pole * 2 * n_items;
+                    if (SV.head.last) vec_update<true>(SA, n, SV.co, SV.head, Up, x, pv, vec_index);
+                    else vec_update<false>(SA, n, SV.co, SV.head, Up, x, pv, vec_index);
                 }
                 s0 = it;
                 k_sync();   // from here the coefficients may be written again
@@ -1155,8 +1158,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 const f32x2 alf = lo_hi(al.x, al.y);
                 const int e = S.e;
                 const uint32_t ubase = smem_addr(U);
-                // two pairs at a time: their loads are in flight together
-                constexpr int kB = 2;
+                // three pairs at a time: their loads are in flight together
+                constexpr int kB = 3;
                 for (int i0 = tid; i0 < n_items; i0 += kB * 32 * nwp) {
                     longlong2 w[kB];
 #pragma unroll
