@@ -29,6 +29,7 @@
 //   increasing in mu; the rules do not depend on mu, so no solve is repeated.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cfloat>
 #include <cstdint>
 #include <type_traits>
@@ -193,10 +194,11 @@ __global__ void __launch_bounds__(1024) k_lanczos(const __grid_constant__ SolveP
     }
 }
 
-// A column of a [K][32] array in shared memory: entry k of this thread's node.
+// A column of a [K][stride] array in shared memory: entry k of this thread's node.
 struct Column {
     double* p;
-    __device__ __forceinline__ double& operator[](int k) const { return p[32 * k]; }
+    int stride;
+    __device__ __forceinline__ double& operator[](int k) const { return p[stride * k]; }
 };
 
 // Eigenvalues and first-row eigenvector components of the n x n Jacobi
@@ -262,9 +264,9 @@ __device__ bool jacobi_eig_first_row(int n, Column d, Column e, Column z) {
 __global__ void __launch_bounds__(32) k_gauss_rules(int n_nodes, const LanczosParams L, double* __restrict__ lambda,
                                                     double* __restrict__ weight) {
     extern __shared__ double cols[];
-    const int j = blockIdx.x * 32 + threadIdx.x;
+    const int nb = (int)blockDim.x, j = blockIdx.x * nb + threadIdx.x;
     if (j >= n_nodes) return;
-    const Column d{cols + threadIdx.x}, e{d.p + 32 * L.K}, z{e.p + 32 * L.K};
+    const Column d{cols + threadIdx.x, nb}, e{d.p + nb * L.K, nb}, z{e.p + nb * L.K, nb};
     const long long base = (long long)j * L.K;
     const int n = L.k_used[j];
     if (n <= 0) {
@@ -427,10 +429,14 @@ cudaError_t launch_lanczos(const SolveParams& P, const LanczosParams& L, int pre
 cudaError_t launch_gauss_rules(int n_nodes, const LanczosParams& L, double* lambda, double* weight,
                                cudaStream_t stream) {
     if (n_nodes <= 0) return cudaSuccess;
-    const size_t smem = (size_t)3 * 32 * L.K * sizeof(double);   // 96 KiB at K = 128
-    const cudaError_t e = cudaFuncSetAttribute(k_gauss_rules, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // Nodes of one warp wait for each other's longer sweeps (the chases of 32
+    // nodes run to the longest, twice the mean), so a warp takes only as many
+    // as keep about four warps an SM.
+    const int nb = std::max(1, std::min(32, (n_nodes + 607) / 608));
+    const size_t smem = (size_t)3 * nb * L.K * sizeof(double);   // 96 KiB at K = 128
+    const cudaError_t e = cudaFuncSetAttribute(k_gauss_rules, cudaFuncAttributeMaxDynamicSharedMemorySize, 98304);
     if (e != cudaSuccess) return e;
-    k_gauss_rules<<<(n_nodes + 31) / 32, 32, smem, stream>>>(n_nodes, L, lambda, weight);
+    k_gauss_rules<<<(n_nodes + nb - 1) / nb, nb, smem, stream>>>(n_nodes, L, lambda, weight);
     return cudaGetLastError();
 }
 
