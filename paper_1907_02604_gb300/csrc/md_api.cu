@@ -119,7 +119,7 @@ void free_ham(Ham& H) {
     void* ptrs[] = {H.V, H.V32, H.atom_xyz, H.atom_depth, H.atom_sigma, H.proj_i0, H.proj_len,
                     H.proj_d, H.proj_g, H.proj_d32, H.proj_g32, H.proj_C, H.proj_absum,
                     H.proj_C32, H.proj_rows, H.pl_ptr, H.pl_atom, H.pl_val32, H.pl_val64, H.proj_fx, H.proj_fxc,
-                    H.scratch, H.lz_buf};
+                    H.scratch, H.lz_buf, H.sync_buf};
     for (void* p : ptrs)
         if (p) cudaFree(p);
 }
@@ -611,6 +611,7 @@ struct md_plan {
     cudaStream_t cap = nullptr;
     bool direct = false;               // launched at creation on `dstream`, temporaries freed stream-ordered
     cudaStream_t dstream = nullptr;
+    bool pooled = false;               // direct, device buffers carved from the handle's
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -642,6 +643,7 @@ void plan_free(md_plan* pl) {
                     pl->d_resid, pl->d_xsrc, pl->d_z, pl->d_w, pl->d_counter};
     for (void* p : ptrs)
         if (p) {
+            if (pl->pooled) continue;   // the handle's
             if (pl->direct) cudaFreeAsync(p, pl->dstream);
             else cudaFree(p);
         }
@@ -944,11 +946,13 @@ cudaError_t plan_capture(md_plan* pl) {
 // direct: launch at once on `stream` without a graph and without
 // synchronising it (device temporaries allocated and freed stream-ordered,
 // uploads staged through the handle's pinned buffers); the caller frees the
-// plan right after.  Otherwise the batch is captured as a graph for replay.
+// plan right after.  pooled (with direct): for a call that waits for its
+// results; the buffers come from the handle and the events time the launch.
+// Otherwise the batch is captured as a graph for replay.
 md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md_nodes* nodes,
                       const md_solver_opts* opts_in, double* rho_out, double* e_out, md_workspace* ckpt,
                       bool borrow_scratch, cudaStream_t stream, md_plan** out,
-                      const FusedArgs* fused = nullptr, bool direct = false) {
+                      const FusedArgs* fused = nullptr, bool direct = false, bool pooled = false) {
     *out = nullptr;
     md_status st = check_device();
     if (st != MD_OK) return st;
@@ -984,6 +988,7 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     pl->own_scratch = !borrow_scratch;
     pl->multishift = ms;
     pl->direct = direct;
+    pl->pooled = pooled;
     pl->dstream = stream;
     std::memset(&pl->P, 0, sizeof(pl->P));
     auto fail = [&](md_status s) {
@@ -997,7 +1002,7 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
             return fail(set_error((_e == cudaErrorMemoryAllocation) ? MD_ERR_OOM : MD_ERR_CUDA, \
                                   std::string("CUDA: ") + cudaGetErrorString(_e) + " (" #expr ")")); \
     } while (0)
-    PTRY(cudaStreamCreateWithFlags(&pl->cap, cudaStreamNonBlocking));
+    if (!direct) PTRY(cudaStreamCreateWithFlags(&pl->cap, cudaStreamNonBlocking));
     PTRY(cudaEventCreate(&pl->ev0));
     PTRY(cudaEventCreate(&pl->ev1));
     if (n_sys == 0) {
@@ -1038,7 +1043,25 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
                      kry_scale(H) > 0.0 && kry_classes(H, R, korder, kfirst, kshape, kdims);
     const bool kvec = ckpt || fused;   // the solution vectors are needed
     const size_t kneed = kry ? kry_params(H, kfirst, kshape, kdims, pl->kry, kvec ? Pn : 0, !ckpt) : 0;
+    if (direct && !kry) PTRY(cudaStreamCreateWithFlags(&pl->cap, cudaStreamNonBlocking));   // for tuning trials
+    size_t carved = 0;
+    if (pooled) {
+        const size_t most = n_work * sizeof(SysDesc) + nn * sizeof(NodeDesc) + 2 * Pn * sizeof(double2) +
+                            n_sys * (3 * sizeof(int) + 2 * sizeof(double) + sizeof(double2)) + 16 * 256;
+        if (most > H.sync_bytes) {
+            if (H.sync_buf) cudaFree(H.sync_buf);
+            H.sync_buf = nullptr;
+            H.sync_bytes = 0;
+            PTRY(cudaMalloc(&H.sync_buf, most));
+            H.sync_bytes = most;
+        }
+    }
     auto dmalloc = [&](auto** p, size_t b) {
+        if (pooled) {
+            *(void**)p = (char*)H.sync_buf + carved;
+            carved += (b + 255) / 256 * 256;
+            return cudaSuccess;
+        }
         return direct ? cudaMallocAsync((void**)p, b, stream) : cudaMalloc((void**)p, b);
     };
     PTRY(dmalloc(&pl->d_sys, n_work * sizeof(SysDesc)));
@@ -1251,7 +1274,9 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     }
 
     if (direct) {   // [reset counters, solver, accumulation] on the caller's stream, now
+        if (pooled) PTRY(cudaEventRecord(pl->ev0, stream));
         PTRY(plan_enqueue(pl, stream));
+        if (pooled) PTRY(cudaEventRecord(pl->ev1, stream));
         if (!H.scratch_ev) PTRY(cudaEventCreateWithFlags(&H.scratch_ev, cudaEventDisableTiming));
         PTRY(cudaEventRecord(H.scratch_ev, stream));
         pl->launched = true;
@@ -1339,6 +1364,17 @@ md_status plan_stats(md_plan* pl, cudaStream_t stream, md_stats* stats) {
     return MD_OK;
 }
 
+// One solve enqueued for a call that goes on to read its results (plan_stats)
+// before it returns.  No graph, streams or allocations of its own: preparing
+// and discarding those took 0.4 ms, as long as a small solve.
+md_status plan_solve(const md_hamiltonian* ham, const md_poles* poles, const md_nodes* nodes,
+                     const md_solver_opts* opts, double* rho_out, double* e_out, md_workspace* ckpt,
+                     cudaStream_t stream, md_plan** out, const FusedArgs* fused = nullptr) {
+    const md_status st = plan_create(ham, poles, nodes, opts, rho_out, e_out, ckpt, true, stream, out, fused, true, true);
+    if (st != MD_OK) cudaStreamSynchronize(stream);   // nothing queued still uses the handle's buffers
+    return st;
+}
+
 md_status density_impl(const md_hamiltonian* ham, const md_poles* poles, const md_nodes* nodes,
                        const md_solver_opts* opts, double* rho_out, double* e_out, md_workspace* ckpt,
                        md_stats* stats, cudaStream_t stream) {
@@ -1348,15 +1384,14 @@ md_status density_impl(const md_hamiltonian* ham, const md_poles* poles, const m
         if (pl) plan_free(pl);
         return st;
     }
-    md_status st = plan_create(ham, poles, nodes, opts, rho_out, e_out, ckpt, true, stream, &pl);
+    md_status st = plan_solve(ham, poles, nodes, opts, rho_out, e_out, ckpt, stream, &pl);
     if (st != MD_OK) return st;
     if (pl->n_sys == 0) {
         if (stats) std::memset(stats, 0, sizeof(*stats));
         plan_free(pl);
         return MD_OK;
     }
-    st = plan_launch(pl, stream);
-    if (st == MD_OK) st = plan_stats(pl, stream, stats);
+    st = plan_stats(pl, stream, stats);
     plan_free(pl);
     return st;
 }
@@ -1402,9 +1437,8 @@ md_status free_energy_impl(const md_hamiltonian* ham, const md_poles* poles, con
         MD_TRY_CUDA(cudaMallocAsync((void**)&d_ws, Pn * sizeof(double2), s));
         MD_TRY_CUDA(cudaMemcpyAsync(d_ws, w_entropy, Pn * sizeof(double2), cudaMemcpyHostToDevice, s));
     }
-    st = plan_create(ham, poles, nodes, opts, d_rho, d_e, nullptr, true, s, &pl);
+    st = plan_solve(ham, poles, nodes, opts, d_rho, d_e, nullptr, s, &pl);
     if (st != MD_OK) goto done;
-    if ((st = plan_launch(pl, s)) != MD_OK) goto done;
     st = plan_stats(pl, s, stats);
     if (fatal(st)) goto done;
     if (w_entropy) MD_TRY_CUDA(launch_entropy((int)nn, Pn, pl->d_xsrc, d_ws, kT, d_s, s));
@@ -2352,18 +2386,15 @@ md_status md_density_fused_adjoint(const md_hamiltonian* ham, const md_poles* po
     if (e != cudaSuccess) return set_error(MD_ERR_CUDA, std::string("CUDA: ") + cudaGetErrorString(e));
     FusedArgs fa{dL_dV_out, dL_drho, dL_de, nullptr, nullptr};
     md_plan* pl = nullptr;
-    st = plan_create(ham, poles, nodes, opts, rho_out, e_out, nullptr, true, s, &pl, &fa);
+    st = plan_solve(ham, poles, nodes, opts, rho_out, e_out, nullptr, s, &pl, &fa);
     if (st != MD_OK) return st;
     if (pl->n_sys == 0) {
         if (stats) std::memset(stats, 0, sizeof(*stats));
         plan_free(pl);
         return MD_OK;
     }
-    st = plan_launch(pl, s);
-    md_status st2 = MD_OK;
-    if (st == MD_OK) st2 = plan_stats(pl, s, stats);
+    const md_status st2 = plan_stats(pl, s, stats);
     plan_free(pl);
-    if (st != MD_OK) return st;
     if (st2 == MD_ERR_CUDA || st2 == MD_ERR_INVALID || st2 == MD_ERR_TIMEOUT) return st2;
     if (forces_out) {
         ForceParams F;
@@ -2424,15 +2455,14 @@ md_status md_density_matrix_rows(const md_hamiltonian* ham, const md_poles* pole
     if (o.kernel == 2) o.kernel = 1;   // the row epilogue lives in the generic kernel
     FusedArgs fa{nullptr, nullptr, nullptr, rows_out, d_off};
     md_plan* pl = nullptr;
-    st = plan_create(ham, poles, nodes, &o, rho_out, e_out, nullptr, true, s, &pl, &fa);
+    st = plan_solve(ham, poles, nodes, &o, rho_out, e_out, nullptr, s, &pl, &fa);
     if (st != MD_OK) {
         cudaFree(d_off);
         return st;
     }
     md_status st2 = MD_OK;
     if (pl->n_sys > 0) {
-        st = plan_launch(pl, s);
-        if (st == MD_OK) st2 = plan_stats(pl, s, stats);
+        st2 = plan_stats(pl, s, stats);
     } else if (stats) {
         std::memset(stats, 0, sizeof(*stats));
     }

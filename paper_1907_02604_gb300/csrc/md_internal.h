@@ -82,6 +82,10 @@ struct Ham {
     // cached work lists and per-node Lanczos results of md_lssgq_rules (grow-only)
     void* lz_buf = nullptr;
     size_t lz_bytes = 0;
+    // descriptors and per-system results of synchronous solves (grow-only; a
+    // synchronous call has finished with it when it returns)
+    void* sync_buf = nullptr;
+    size_t sync_bytes = 0;
     // pinned staging of the uploads of asynchronous md_density calls, two in
     // turn; an event marks when a buffer's last uploads have been read
     struct Stage {
