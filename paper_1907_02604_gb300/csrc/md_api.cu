@@ -332,7 +332,7 @@ KryShape kry_shape(const Ham& H, int m0, int m1, int m2, int c, int dev) {
         const double here = std::min(local, per_pt * reach[0] * reach[1] * reach[2]);
         const double rows = here * 3.2 * H.proj_rc * H.proj_rc / (H.h[1] * H.h[2]) * m1 / reach[1] * s.depth / reach[2];
         tables = (size_t)(local * 96);
-        if (u + kry_max_threads() * 32 + 1024 > budget) return s;
+        if (u + kry_max_threads() * 32 + 1024 + 32 * kMaxLocalProjAtoms > budget) return s;
         s.spill = u + tables + (size_t)((std::max(1.1 * rows, 1280.0) + 1.1 * here * (2.0 * H.proj_rc / H.h[0] + 2)) * 16) > budget;
     } else if (u > budget) {
         return s;
@@ -952,7 +952,8 @@ cudaError_t plan_capture(md_plan* pl) {
 md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md_nodes* nodes,
                       const md_solver_opts* opts_in, double* rho_out, double* e_out, md_workspace* ckpt,
                       bool borrow_scratch, cudaStream_t stream, md_plan** out,
-                      const FusedArgs* fused = nullptr, bool direct = false, bool pooled = false) {
+                      const FusedArgs* fused = nullptr, bool direct = false, bool pooled = false,
+                      bool per_pole = false) {
     *out = nullptr;
     md_status st = check_device();
     if (st != MD_OK) return st;
@@ -994,6 +995,15 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     auto fail = [&](md_status s) {
         plan_free(pl);
         return s;
+    };
+    // the solution vectors of the node-shared kernel can take more scratch than
+    // the per-pole kernels' slots: where it cannot be had, those run
+    auto retry_per_pole = [&]() {
+        cudaGetLastError();
+        plan_free(pl);
+        if (pooled) cudaStreamSynchronize(stream);
+        return plan_create(ham, poles, nodes, opts_in, rho_out, e_out, ckpt, borrow_scratch, stream, out, fused, direct,
+                           pooled, true);
     };
 #define PTRY(expr)                                                                          \
     do {                                                                                    \
@@ -1037,9 +1047,12 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     std::vector<int> korder, kfirst;
     std::vector<KryShape> kshape;
     std::vector<NodeDesc> kdims;
-    // (mixed shifted COCG keeps its FP32 kernel: it needs no more than FP32 moves a step)
-    const bool kry = opts.kernel == 0 && opts.block == 0 && opts.ctas_per_sm == 0 && Pn <= kKryMaxPoles &&
-                     !(ms && opts.precision == MD_PREC_MIXED) &&
+    // (mixed shifted COCG keeps its FP32 kernel, a step of which is as fast and
+    // one sequence a node too; a single pole in mixed precision has nothing to
+    // share: 34 G complex FP32 point-iterations a second against 26 G real
+    // fixed-point ones on the bulk cell)
+    const bool kry = !per_pole && opts.kernel == 0 && opts.block == 0 && opts.ctas_per_sm == 0 && Pn <= kKryMaxPoles &&
+                     (Pn > 1 || opts.precision == MD_PREC_FP64) && !(ms && opts.precision == MD_PREC_MIXED) &&
                      kry_scale(H) > 0.0 && kry_classes(H, R, korder, kfirst, kshape, kdims);
     const bool kvec = ckpt || fused;   // the solution vectors are needed
     const size_t kneed = kry ? kry_params(H, kfirst, kshape, kdims, pl->kry, kvec ? Pn : 0, !ckpt) : 0;
@@ -1199,12 +1212,16 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
             if (H.scratch) cudaFree(H.scratch);
             H.scratch = nullptr;
             H.scratch_bytes = 0;
-            PTRY(cudaMalloc(&H.scratch, need));
+            const cudaError_t e = cudaMalloc(&H.scratch, need);
+            if (e == cudaErrorMemoryAllocation && kry) return retry_per_pole();
+            PTRY(e);
             H.scratch_bytes = need;
         }
         pl->scratch = H.scratch;
     } else {
-        PTRY(cudaMalloc(&pl->scratch, need));
+        const cudaError_t e = cudaMalloc(&pl->scratch, need);
+        if (e == cudaErrorMemoryAllocation && kry) return retry_per_pole();
+        PTRY(e);
     }
     P.scratch = (char*)pl->scratch;
     if (kry) {
@@ -1369,8 +1386,9 @@ md_status plan_stats(md_plan* pl, cudaStream_t stream, md_stats* stats) {
 // and discarding those took 0.4 ms, as long as a small solve.
 md_status plan_solve(const md_hamiltonian* ham, const md_poles* poles, const md_nodes* nodes,
                      const md_solver_opts* opts, double* rho_out, double* e_out, md_workspace* ckpt,
-                     cudaStream_t stream, md_plan** out, const FusedArgs* fused = nullptr) {
-    const md_status st = plan_create(ham, poles, nodes, opts, rho_out, e_out, ckpt, true, stream, out, fused, true, true);
+                     cudaStream_t stream, md_plan** out, const FusedArgs* fused = nullptr, bool per_pole = false) {
+    const md_status st =
+        plan_create(ham, poles, nodes, opts, rho_out, e_out, ckpt, true, stream, out, fused, true, true, per_pole);
     if (st != MD_OK) cudaStreamSynchronize(stream);   // nothing queued still uses the handle's buffers
     return st;
 }
@@ -1437,7 +1455,11 @@ md_status free_energy_impl(const md_hamiltonian* ham, const md_poles* poles, con
         MD_TRY_CUDA(cudaMallocAsync((void**)&d_ws, Pn * sizeof(double2), s));
         MD_TRY_CUDA(cudaMemcpyAsync(d_ws, w_entropy, Pn * sizeof(double2), cudaMemcpyHostToDevice, s));
     }
-    st = plan_solve(ham, poles, nodes, opts, d_rho, d_e, nullptr, s, &pl);
+    // The entropy weights cancel, so that s_j shows how far a mixed x_jp(j) is
+    // from its exact value (2e-9 with the per-pole solver): mixed calls with an
+    // entropy keep that solver and its values.
+    st = plan_solve(ham, poles, nodes, opts, d_rho, d_e, nullptr, s, &pl, nullptr,
+                    w_entropy && opts && opts->precision == MD_PREC_MIXED);
     if (st != MD_OK) goto done;
     st = plan_stats(pl, s, stats);
     if (fatal(st)) goto done;
@@ -2455,7 +2477,9 @@ md_status md_density_matrix_rows(const md_hamiltonian* ham, const md_poles* pole
     if (o.kernel == 2) o.kernel = 1;   // the row epilogue lives in the generic kernel
     FusedArgs fa{nullptr, nullptr, nullptr, rows_out, d_off};
     md_plan* pl = nullptr;
-    st = plan_solve(ham, poles, nodes, &o, rho_out, e_out, nullptr, s, &pl, &fa);
+    // (rows of mixed solves are within tol / Im z, 1e-9, of the exact ones: they
+    // keep the per-pole solver and its values)
+    st = plan_solve(ham, poles, nodes, &o, rho_out, e_out, nullptr, s, &pl, &fa, o.precision == MD_PREC_MIXED);
     if (st != MD_OK) {
         cudaFree(d_off);
         return st;

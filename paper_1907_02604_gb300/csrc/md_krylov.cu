@@ -660,14 +660,9 @@ struct PoleState {
     double gr, gi;     // x(j) * scale
     double rn;         // ||r||
     int conv;          // step at which ||r|| <= tol
-    int frz;           // step at which the solution vector is complete (||r|| <= kFreeze tol)
     double cr, ci;     // chi = zeta / ||u||
     double mr, mi;     // m of the last step of the chunk before
 };
-// Solution vectors are carried on until ||r|| <= 0.3 tol: the other poles of
-// the node go on anyway, and the slowest pays a few steps.
-constexpr double kFreeze = 0.3;
-
 __device__ __forceinline__ void pole_step(PoleState& s, double a, double b2, bool sum) {
     const double dr = a - s.zr - s.er, di = -s.zi - s.ei;
     const double inv = 1.0 / (dr * dr + di * di);
@@ -708,7 +703,7 @@ __device__ void vec_coefs(const VecHist* hist, int n, int s0, PoleState& s, int 
         }
         for (int j = n - 1; j >= 0; --j) {
             const VecHist h = hist[(size_t)j * kKryMaxPoles + pole];
-            const bool on = s.frz == 0 || s0 + 1 + j <= s.frz;
+            const bool on = s.conv == 0 || s0 + 1 + j <= s.conv;   // a solution ends where its pole met tol
             const double2 c = on ? h.c : make_double2(0.0, 0.0);
             if (j == n - 1) {
                 w = c;
@@ -733,9 +728,9 @@ __device__ void vec_coefs(const VecHist* hist, int n, int s0, PoleState& s, int 
             head->sv = sv;
             head->om = make_double2(-(s.mr * w.x - s.mi * w.y), -(s.mr * w.y + s.mi * w.x));
             head->nu = make_double2(-(s.mr * v.x - s.mi * v.y), -(s.mr * v.y + s.mi * v.x));
-            head->act = s.frz == 0 || s.frz > s0;
+            head->act = s.conv == 0 || s.conv > s0;
             head->first = s0 == 0;
-            head->last = s.frz != 0;
+            head->last = s.conv != 0;
         }
     }
     const double2 m = hist[(size_t)(n - 1) * kKryMaxPoles + pole].m;
@@ -945,7 +940,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         if (scalar_warp && rank == 0 && P.K == 0) {
             for (int k = lane; k < P.P; k += 32, ++np) {
                 const double2 z = P.z[k];
-                ps[np] = PoleState{(z.x - P.shift) / P.scale, z.y / P.scale, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0, 1.0, 0, 0, 8.0, 0.0,
+                ps[np] = PoleState{(z.x - P.shift) / P.scale, z.y / P.scale, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0, 1.0, 0, 8.0, 0.0,
                                    0.0, 0.0};
             }
         }
@@ -960,12 +955,12 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
             return ((long long)(z0 + d) * m1 + pb) * m0 + 2 * (pc - pb * npx);
         };
         // Pole recurrences of step k (the scalar warp of rank 0); true once
-        // nothing is left to do.  x_jp(j) sums up to the step after the one
-        // at which all poles met tol, whether or not vectors are carried on.
+        // all have met tol.  x_jp(j) sums up to the step after that, whether or
+        // not vectors are kept.
         int proc = 0, g_stop = 0;
         bool all_done = false;
         auto poles = [&](int step) {
-            bool all = true, done = true;
+            bool all = true;
             const double p2 = __hiloint2double((1023 + S.e_hat) << 20, 0);
             for (int k = 0; k < np; ++k) {
                 PoleState& s = ps[k];
@@ -985,15 +980,12 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                     s.rn = rn;
                     if (rn <= P.tol) s.conv = step;
                 }
-                if (!s.frz && rn <= kFreeze * P.tol) s.frz = step;
                 all = all && s.conv;
-                done = done && s.frz;
             }
             all = __all_sync(0xffffffffu, all);
-            done = __all_sync(0xffffffffu, done);
             if (all && !g_stop) g_stop = step + 1;
             proc = step;
-            all_done = P.vec ? all && done : all;
+            all_done = all;
         };
         int s0 = 0;   // steps the solution vectors hold
         int it = 0, stop = bad ? 1 : 0;
