@@ -59,6 +59,7 @@ namespace {
 constexpr int kMaxThreads = 19 * 32 + 32;   // 20 warps: 96 registers a thread
 constexpr int kMaxWarps = kMaxThreads / 32;
 constexpr int kMaxC = 8;
+constexpr int kMeasure = -1;   // KShared::stop: sum ||w - alpha u||^2 first
 
 __device__ __forceinline__ uint32_t k_rank() {
     uint32_t r;
@@ -190,7 +191,7 @@ struct KChunk {      // up to kKryChunkRows rows of one atom
 
 struct KShared {
     long long part[kMaxWarps][4];
-    long long mbox[kMaxC][5];     // per rank: u.w (2), w.w (2), stop flag of rank 0
+    long long mbox[kMaxC][7];     // per rank: u.w (2), w.w (2), stop flag of rank 0, ||w - alpha u||^2 (2)
     int2 ca, cg;                  // alpha and g as limbs
     int e;                        // u_new = (w - alpha u) 2^e
     int zlo[kMaxC + 1];           // first plane of each rank's slab
@@ -198,6 +199,7 @@ struct KShared {
     int work;
     // scalar warp's state
     double s0, inv0;              // ||u||^2, 1/||u||^2
+    double drift;                 // bound of the relative error of s0
     double a_hat, b2_hat;         // alpha, beta^2 of the step just taken (in units of scale)
     double scale0;                // Lanczos breakdown scale
     int e_hat;                    // its e
@@ -929,6 +931,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 U[(src_z - z0 + Q) * pp + b * pitch + a] = split31(1LL << 59);
             S.s0 = 0x1p-6;
             S.inv0 = 0x1p6;
+            S.drift = 0x1p-53;
             S.cg = make_int2(0, 0);
             S.stop = 0;
             S.a_hat = 0.0;
@@ -1055,7 +1058,35 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 const double s1 = (double)t[0] * 0x1p-62 + (double)t[1] * 0x1p-83;
                 const double s2 = (double)t[2] * 0x1p-62 + (double)t[3] * 0x1p-82;
                 const double al = s1 * S.inv0;
-                double n2 = s2 - s1 * al;
+                double n2 = s2 - s1 * al, err = 0x1p-53 * s2;
+                // An error d of ||u||^2 makes one of d alpha^2 / beta^2 in the
+                // next: it dies out while |alpha| < beta and grows step by step
+                // where the potential dominates H.  Beyond 2^-49 the norm is
+                // summed instead (one more pass over w and u; no step of the
+                // usual Hamiltonians needs it).
+                err += al * al * S.drift * S.s0;
+                if (!flag && !(err <= 0x1p-49 * n2)) {
+                    const double top = fmax(n2, 0x1p-40 * s2);
+                    const int e = min(40, (-4 - (((__double2hiint(top) >> 20) & 0x7ff) - 1022)) >> 1);
+                    const int2 ca = to_limbs(al);
+                    __syncwarp();
+                    if (lane == 0) {
+                        S.ca = ca;
+                        S.e = e;
+                        S.stop = kMeasure;
+                    }
+                    __syncthreads();
+                    __syncthreads();
+                    const bool on = lane < nwp;
+                    const long long s = warp_sum4(on ? S.part[lane][0] : 0LL, on ? S.part[lane][1] : 0LL, 0LL, 0LL, lane);
+                    if ((lane & 2) == 0 && (lane >> 2) < C)
+                        k_st_remote(k_map(smem_addr(&S.mbox[rank][5 + (lane & 1)]), lane >> 2), s);
+                    k_sync();
+                    long long hh = 0, l = 0;
+                    for (int r = 0; r < C; ++r) hh += S.mbox[r][5], l += S.mbox[r][6];
+                    n2 = ldexp((double)hh * 0x1p-62 + (double)l * 0x1p-82, -2 * e);
+                    err = 0x1p-53 * n2;
+                }
                 if (!(n2 > 0.0)) n2 = 0.0;
                 const double b2 = n2 * S.inv0;
                 int st = flag;
@@ -1090,7 +1121,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 const double p2 = __hiloint2double((1023 + e) << 20, 0);   // 2^e
                 const double s0n = n2 * p2 * p2;
                 const int2 cg = to_limbs(n2 * p2 * S.inv0);
-                const double inv = 1.0 / s0n;
+                const double inv = 1.0 / s0n, drift = err * p2 * p2 * inv;
                 __syncwarp();
                 if (lane == 0) {
                     S.a_hat = al;
@@ -1100,11 +1131,37 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                         S.cg = cg;
                         S.s0 = s0n;
                         S.inv0 = inv;
+                        S.drift = drift;
                     }
                 }
                 __syncwarp();
             } else {
                 __syncthreads();
+                if (S.stop == kMeasure) {
+                    const int2 al = S.ca;
+                    const f32x2 alf = lo_hi(al.x, al.y);
+                    const int e = S.e;
+                    Dots sq;
+#pragma unroll 1
+                    for (int item = tid; item < n_items; item += 32 * nwp) {
+                        const int d = (int)fdiv((uint32_t)item, SA.div_pc), pc = item - d * npc;
+                        const int pb = (int)fdiv((uint32_t)pc, div_px);
+                        const int4 u = *reinterpret_cast<const int4*>(U + (d + Q) * pp + pb * pitch + 2 * (pc - pb * npx));
+                        const longlong2 w = Wp[item];
+                        const int ax = opaque(al.x);
+                        Acc a0, a1;
+                        a0.mac(u.x, hi_lo(u.x, u.y), ax, alf);
+                        a1.mac(u.z, hi_lo(u.z, u.w), ax, alf);
+                        const long long t0 = w.x - a0.fold(), t1 = w.y - a1.fold();
+                        sq.add(0, 0, split31(e >= 0 ? t0 << e : t0 >> -e));
+                        sq.add(0, 0, split31(e >= 0 ? t1 << e : t1 >> -e));
+                    }
+                    const long long s = warp_sum4(sq.hh2, sq.l2(), 0LL, 0LL, lane);
+                    if (lane < 2) S.part[warp][lane] = s;
+                    __syncthreads();
+                    k_sync();
+                    __syncthreads();
+                }
             }
             stop = S.stop;
             if (P.vec && (stop || it % kKryVec == 0)) {
