@@ -5,8 +5,8 @@ One step = one pass of the path over one batch of nodes of the bulk
 workload (1,024-atom hcp Mg-like cell, 96x96x160 grid, 8th-order FD,
 Gaussian projectors, P = 16 poles, 33^3 regions, mixed precision): Fermi
 poles on the spectral interval, the cost-sorted work list, every
-(node, pole) COCG solve, and the pole-weighted density and band-energy
-accumulation.  Successive steps take successive node batches of the
+(node, pole) solve (one real Krylov sequence per node for all its poles),
+and the pole-weighted density and band-energy accumulation.  Successive steps take successive node batches of the
 workload (4,096 nodes in all).
 
 Prints one JSON line (rank 0):
@@ -15,10 +15,11 @@ Prints one JSON line (rank 0):
   e2e      the same metric through the C ABI from host buffers: every step
            builds the Hamiltonian from host arrays, solves, and copies rho
            and e back to the host;
-  roofline HBM roofline of the solver kernel: algorithmic bytes (80 B per
-           region point per COCG iteration in mixed mode, 160 B in FP64)
-           / the kernel's CUDA-event time, against the measured copy
-           bandwidth;
+  roofline of the solver kernel: wide integer multiply-adds (24.4 per
+           region point and Krylov step) / the kernel's CUDA-event time,
+           against their measured rate; with --kernel or --block (a per-pole
+           kernel) the HBM roofline, 80 B per region point and COCG iteration
+           in mixed mode, 160 B in FP64;
   cpu_baseline  the FP64 oracle (plain C, OpenMP) on a bounded sample.
 --impl reference times the oracle itself as the reference arm.
 """
@@ -54,6 +55,13 @@ TRAFFIC_FINGERPRINT = "53842885215939a9:0a35456717bedd0f:6685de8068da134b:6a946d
 # pairs x 6 = 72, diagonal 8, projector apply 24 and coefficients 12 (1.5
 # atoms per point), p update 8, x and r updates 16, r^T r and ||r||^2 8, p^T Ap 8
 FP64_FLOPS_PER_POINT_ITER = 156.0
+# The node-shared kernel: hi x hi products (IMAD.WIDE) per region point and
+# real Krylov step at 8th order with projectors: 12 stencil pairs, diagonal,
+# previous vector, alpha, u.w, w.w = 17, and 5 for each of 1.48 projector
+# atoms a point (3 projections, 2 in the apply).  Their rate with distinct
+# operands, 31 a clock and SM, was measured with a probe kernel.
+WIDE_PER_POINT_STEP = 24.4
+WIDE_PER_CLOCK_SM = 31.0
 L2_FLUSH_BYTES = 256 << 20   # written between timed steps: twice the 129 MB L2
 NOMINAL_HBM_GBS = 7900.0   # GB300 HBM3e, vendor figure (context beside the measured copy peak)
 
@@ -476,6 +484,18 @@ def main():
     value = total_solves / (el_ms / 1e3)
     kernel_ms = sum(s["kernel_ms"] for s in stats)
     point_iters = sum(s["total_point_iters"] for s in stats)
+    # the default route runs one real Krylov sequence per node, as long as its
+    # slowest pole's
+    shared = (args.kernel == "auto" and not args.block and not args.ctas_per_sm
+              and (args.method == "cocg" or prec == "fp64"))
+
+    def point_steps_of(plan, i):
+        idx = batch_idx(i)
+        return float((plan.system_info(stream)[1].reshape(-1, w.n_poles).max(axis=1)
+                      * w.region_points()[idx]).sum())
+
+    point_steps = (sum(point_steps_of(plan_of(args.warmup + i), args.warmup + i) for i in range(args.steps))
+                   if shared else None)
     conv = sum(s["n_converged"] for s in stats)
     B = BYTES_PER_POINT_ITER[prec]
     achieved = point_iters * B / (kernel_ms / 1e3) / 1e9
@@ -530,17 +550,19 @@ def main():
                        "method 1: per node one Krylov sequence serves all poles (density only)")
     if prec == "mixed" and not args.no_fp64_form:
         fp64_form = side(_replace(opts, precision="fp64", block=0, ctas_per_sm=0),
-                         "per-pole COCG with FP64 vectors; speedup = value / this value")
+                         "the same sequence without the mixed form's FP64 recomputation of the last step" if shared
+                       else "per-pole COCG with FP64 vectors; speedup = value / this value")
         fp64_form["speedup_mixed_over_fp64"] = value / fp64_form["value"]
-        # its roofline: FP64 operations per region-point iteration over the
+        # per-pole kernel: its roofline: FP64 operations per region-point iteration over the
         # solver kernel's time, against this GPU's FP64 FMA rate measured now
         # (md_fma_rate: bounded FMA chains on every SM)
-        from paper_1907_02604_gb300 import fma_rate
-        peak64 = fma_rate("fp64", stream)
-        ach64 = FP64_FLOPS_PER_POINT_ITER * fp64_form["point_iters"] / (fp64_form["kernel_ms"] / 1e3) / 1e12
-        fp64_form["roofline"] = {"bound": "fp64", "achieved": ach64, "peak": peak64, "unit": "TFLOP/s",
-                                 "frac": ach64 / peak64, "flops_per_point_iter": FP64_FLOPS_PER_POINT_ITER,
-                                 "peak_kind": "measured (md_fma_rate, FP64 FMA chains)"}
+        if not shared:
+            from paper_1907_02604_gb300 import fma_rate
+            peak64 = fma_rate("fp64", stream)
+            ach64 = FP64_FLOPS_PER_POINT_ITER * fp64_form["point_iters"] / (fp64_form["kernel_ms"] / 1e3) / 1e12
+            fp64_form["roofline"] = {"bound": "fp64", "achieved": ach64, "peak": peak64, "unit": "TFLOP/s",
+                                     "frac": ach64 / peak64, "flops_per_point_iter": FP64_FLOPS_PER_POINT_ITER,
+                                     "peak_kind": "measured (md_fma_rate, FP64 FMA chains)"}
 
     # ---- side measurement: the batched uneven workload, all 1,250 nodes x
     # 16 poles (20,000 systems, regions 17^3..41^3) in one graph launch ----
@@ -726,6 +748,22 @@ def main():
         for j in sorted({(args.warmup + i) % n_plans for i in range(args.steps)}):
             timed.append((batch_idx(j), plans[j].rho.cpu().numpy(), plans[j].e.cpu().numpy()))
         cpu, parity = oracle_sample(w, timed, 1e-5 if prec == "mixed" else 1e-6)
+    if shared:
+        n_ops = point_steps * WIDE_PER_POINT_STEP
+        ach = n_ops / (kernel_ms / 1e3) / 1e12
+        mhz = clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or 0.0
+        pk = WIDE_PER_CLOCK_SM * n_sm * mhz * 1e6 / 1e12
+        roofline = {"bound": "integer multiply-add (IMAD.WIDE) issue", "achieved": ach, "peak": pk, "unit": "T mad/s",
+                    "frac": ach / pk if pk else None, "kernel": "k_krylov", "mads_per_point_step": WIDE_PER_POINT_STEP,
+                    "point_steps_per_s": point_steps / (kernel_ms / 1e3), "traffic": None,
+                    "peak_kind": "31 a clock and SM (probe kernel, distinct operands) x SMs x the sampled SM clock"}
+    else:
+        roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                    "frac": achieved / peak, "traffic": traffic,
+                    "frac_of_nominal": achieved / NOMINAL_HBM_GBS, "nominal_peak": NOMINAL_HBM_GBS,
+                    "algorithmic_bytes_per_launch": point_iters * B / len(stats),
+                    "kernel": "k_cocg<MixedMode>" if prec == "mixed" else "k_cocg<FP64Mode>",
+                    "bytes_per_point_iter": B, "peak_kind": peak_kind}
     out = {
         "metric": METRIC,
         "value": value,
@@ -737,7 +775,7 @@ def main():
         "higher_is_better": True,
         "scaling": "weak",
         "vs_baseline": None,
-        "dtype": "f32+f64" if prec == "mixed" else "f64",
+        "dtype": "fixed point 62 bit + f64" if shared else ("f32+f64" if prec == "mixed" else "f64"),
         "data": "synthetic",
         "config": {**workload_config(w, bs, prec),
                    "l2": f"flushed between timed steps ({L2_FLUSH_BYTES >> 20} MB written)",
@@ -749,12 +787,7 @@ def main():
         "iters_mean": float(np.mean([s["iters_mean"] for s in stats])),
         "refreshes_per_system": float(sum(s["reliable_updates"] for s in stats) / max(solves_rank, 1)),
         "point_iters_per_s": point_iters * world / (el_ms / 1e3),
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak, "traffic": traffic,
-                     "frac_of_nominal": achieved / NOMINAL_HBM_GBS, "nominal_peak": NOMINAL_HBM_GBS,
-                     "algorithmic_bytes_per_launch": point_iters * B / len(stats),
-                     "kernel": "k_cocg<MixedMode>" if prec == "mixed" else "k_cocg<FP64Mode>",
-                     "bytes_per_point_iter": B, "peak_kind": peak_kind},
+        "roofline": roofline,
         "cpu_baseline": cpu,
         "parity": parity,
         "gather": gathered,

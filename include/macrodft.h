@@ -118,18 +118,28 @@ typedef struct {
     double tol;            /* stop when ||r||_2 <= tol (||e_j|| = 1); > 0 */
     int32_t maxit;         /* iteration cap per system, > 0 */
     int32_t precision;     /* md_precision */
-    int32_t reliable_every;/* mixed: max iterations between FP64 residual
-                              recomputations (0 = 300) */
-    double reliable_delta; /* mixed: also recompute when ||r|| fell by this
-                              factor since the last one (0 = 3e-3); a refresh
-                              that finds the residual larger than at the
-                              previous one restarts the Krylov recurrence */
+    int32_t reliable_every;/* mixed, per-pole kernels: max iterations between
+                              FP64 residual recomputations (0 = 300) */
+    double reliable_delta; /* mixed, per-pole kernels: also recompute when ||r||
+                              fell by this factor since the last one (0 = 3e-3);
+                              a refresh that finds the residual larger than at
+                              the previous one restarts the Krylov recurrence.
+                              The node-shared kernel recomputes its last step in
+                              FP64 once per node and adds the defect it finds to
+                              every residual before it declares convergence */
     double timeout_s;      /* device wall-clock budget for the call, 0 = none */
-    int32_t block;         /* threads per CTA; 0 = library choice (autotuned) */
+    int32_t block;         /* threads per CTA; 0 = library choice */
     int32_t ctas_per_sm;   /* resident CTAs per SM; 0 = library choice.  With
                               kernel 3: CTAs per cluster (1..8; 0 = the fewest
                               whose slabs fit in shared memory) */
-    int32_t kernel;        /* with block > 0: 0 or 1 = generic kernel, 2 = shared-memory
+    int32_t kernel;        /* 0 with block = 0 and ctas_per_sm = 0: one real Krylov
+                              sequence per node, in 62-bit fixed point, serves all
+                              its poles (fd_order <= 8, P <= 64, no whole-axis
+                              rings, regions that fit a cluster's shared memory,
+                              about 43^3; mixed shifted solves excepted); the
+                              per-pole iterates, residuals and iteration counts are
+                              COCG's.  Other calls autotune the per-pole kernels.
+                              With block > 0: 0 or 1 = generic kernel, 2 = shared-memory
                               z-march kernel (mixed precision, 4th/8th order, no
                               whole-axis rings; ceil(m0*m1/block) <= 4).
                               3 = cluster kernel (block may be 0): mixed precision,
@@ -138,8 +148,8 @@ typedef struct {
                               whose CTAs hold z-slabs of the Krylov vectors p and r
                               in shared memory (halo planes read from the
                               neighbouring CTAs), so the vectors do not stream
-                              through HBM.  With kernel 0 and block 0 the
-                              autotuner includes it among its candidates. */
+                              through HBM.  The autotuner includes it among its
+                              candidates. */
     int32_t method;        /* 0 = one COCG per (node, pole) system.
                               1 = shifted COCG: per node one Krylov sequence, seeded
                               with the pole nearest the real axis, serves all P poles
@@ -163,7 +173,8 @@ typedef struct {
     double iters_mean;
     int64_t total_iters;       /* sum over systems */
     int64_t total_point_iters; /* sum over systems of iters * region points */
-    int64_t reliable_updates;  /* mixed: FP64 residual recomputations */
+    int64_t reliable_updates;  /* mixed: FP64 residual recomputations, summed over
+                                  systems (node-shared kernel: one per system) */
     double max_resid;          /* max final relative residual */
     double kernel_ms;          /* device time of the solver launch */
 } md_stats;

@@ -72,7 +72,8 @@ class SolverOptions:
     timeout_s: float = 0.0
     block: int = 0
     ctas_per_sm: int = 0
-    # "auto" (autotuned), "generic" or "zmarch" (both need block > 0), or
+    # "auto" (one Krylov sequence per node for all its poles where it applies,
+    # else the autotuned per-pole kernels), "generic" or "zmarch" (both need block > 0), or
     # "cluster": Krylov vectors in shared memory, one thread-block cluster per
     # system (mixed precision); there ctas_per_sm is the CTAs per cluster
     # (0 = the fewest whose slabs fit) and block the threads per CTA (0 = auto)

@@ -15,34 +15,39 @@
 // sum_p 4,560 complex iterations.
 //
 // Precision.  The recurrence must hold FP64-like accuracy over a thousand
-// steps (FP32 vectors lose the density at 1e-5), and this part issues 1.6
-// FP64 FMAs per clock and SM against 64 integer multiply-adds into 64 bits
-// (measured).  So the vectors are 62-bit fixed point: a value u in
-// (-1/2, 1/2) is hi 2^-31 + lo 2^-62 with two signed 31-bit limbs, products
-// are exact 32 x 32 -> 64-bit integer multiply-adds kept as two 64-bit sums
-// (hi hi, and hi lo + lo hi; the lo lo terms, below 2^-62, are dropped), and
-// each result is rounded once to 2^-62.  Vectors are kept at norm
-// [1/4, 1/2) by exact powers of two, so the rounding is ~1e-16 of the norm
-// per step, the size of FP64's.  A = (H_R - shift) / scale has ||A|| < 1/2,
-// which bounds every sum below the 64-bit range.  Integer sums are exact and
-// independent of order: the result is bitwise reproducible.
+// steps (FP32 vectors lose the density at 1e-5), and this part issues 1.7
+// FP64 FMAs per clock and SM against 31 integer multiply-adds into 64 bits
+// and 115 FP32 FMAs (measured).  So the vectors are 62-bit fixed point: a
+// value u is hi 2^-31 + lo 2^-62 with two signed 31-bit limbs.  Of a product,
+// hi hi is exact in a 64-bit integer sum and the mixed terms, 2^-31 of it,
+// are FP32 (2^-55 of the product); the lo lo term, below 2^-62, is dropped,
+// except in w.w, where it adds up.  Each result is rounded once to 2^-62.
+// Vectors are kept at norm [1/8, 1/4) by exact powers of two, so the rounding
+// is ~1e-16 of the norm per step, the size of FP64's.  A = (H_R - shift) /
+// scale has ||A|| < 1/2, which bounds every sum below the 64-bit range.
+// ||u||^2 comes from the recurrence (see the step); where |alpha| exceeds beta
+// an error of it would grow, and the norm is summed.
 //
 // Layout.  A thread-block cluster works on one node.  The region is cut into
 // z-slabs, one per CTA; each CTA holds its slab of the current vector u and
 // Q halo planes on either side in shared memory (rows Q zeros apart, so that
-// x neighbours need no bounds checks).  A thread marches its (x, y) columns
-// along z with the 2Q+1 stencil values in registers.  The previous vector,
-// the new one and V are touched by their own thread only, coalesced, in a
-// per-CTA scratch slot that stays in L2.  Per step:
-//   dot    projections on the local projector tables (warp per 32 rows)
-//   A      w = A u - g u_prev                (stencil while the cluster
-//                                             exchanges the projections)
-//   A2     w += nonlocal term, u.w, w.w
+// x neighbours need no bounds checks).  A thread takes pairs of points along
+// x.  The previous vector, the new one, V and the projector rows that cover a
+// pair are touched by their own thread only, coalesced, in a per-CTA scratch
+// slot that stays in L2.  Per step:
+//   dot    projections on the local projector tables, summed over the cluster
+//   A      w = A u - g u_prev with the nonlocal term, u.w, w.w
 //          one exchange of u.w and w.w: alpha = u.w / u.u, and
 //          ||w - alpha u||^2 = w.w - alpha u.w gives beta in the same one
 //   B      u_new = (w - alpha u) 2^e, halo planes pushed to the neighbours
 // One warp of each CTA computes no points: it sums the partials, and in
 // rank 0 it runs the pole recurrences of step k-1 during step k.
+//
+// Bound: instruction issue and latency at 20 warps an SM (19 computing, 96
+// registers): 255 instructions a point-step without projectors, 560 with
+// them, at 1.9 and 1.7 issued a clock.  96 nodes x 16 poles on 33^3 regions
+// with projectors take 108 ms, 506 with one complex COCG per pole in mixed
+// precision; 13 nodes x 16 poles on 25^3 in FP64 9.1 ms against 278.
 #include <cuda_runtime.h>
 
 #include <cfloat>
