@@ -47,11 +47,10 @@ __device__ __forceinline__ double min_image(double d, double L, int periodic) {
     return periodic ? d - L * rint(d / L) : d;
 }
 
-// Visit every atom in the cells around grid point (ix, iy, iz).
+// Visit every entry of the cell list in the cells around grid point (ix, iy, iz).
 template <class F>
 __device__ __forceinline__ void for_each_near_atom(const GridGeo& g, const int* nc, const double* cell,
-                                                   const int* cstart, const int* catoms, int ix,
-                                                   int iy, int iz, F&& f) {
+                                                   const int* cstart, int ix, int iy, int iz, F&& f) {
     const int pc[3] = {min(max((int)floor(ix * g.h[0] / cell[0]), 0), nc[0] - 1),
                        min(max((int)floor(iy * g.h[1] / cell[1]), 0), nc[1] - 1),
                        min(max((int)floor(iz * g.h[2] / cell[2]), 0), nc[2] - 1)};
@@ -78,7 +77,7 @@ __device__ __forceinline__ void for_each_near_atom(const GridGeo& g, const int* 
                 if (g.periodic[0] && nc[0] >= 3) wx = (cx + nc[0]) % nc[0];
                 else if (wx < 0 || wx >= nc[0]) continue;
                 const int c = wx + nc[0] * (wy + nc[1] * wz);
-                for (int e = cstart[c]; e < cstart[c + 1]; ++e) f(catoms[e]);
+                for (int e = cstart[c]; e < cstart[c + 1]; ++e) f(e);
             }
         }
     }
@@ -91,143 +90,68 @@ struct CellArgs {
     const int* atoms;
 };
 
-// Wells summed over a tile of 32 x 8 x 8 points per block.  The Gaussian is a
-// product of three 1-D factors, so each atom near the tile needs only 48
-// exponentials and squared displacements, kept in shared memory; a point and
-// atom then cost an addition, a comparison and a multiply-add in FP64 (the
-// scarce pipe here: 1.7 a clock and SM), and columns outside the sphere are
-// skipped.  One exponential and three minimum-image divisions per point and
-// atom took 21 ms on the 96 x 96 x 160 grid with 1,024 atoms.
-constexpr int kTx = 32, kTy = 8, kTz = 8;      // tile
-constexpr int kTab = kTx + kTy + kTz;
-constexpr int kAtomBatch = 16;                 // atoms tabulated at a time
-constexpr int kNear = 512;                     // atoms of the list in shared memory
-
-// Lower bound of the squared distance from X to the points lo..hi (grid
-// indices) on one axis.
-__device__ __forceinline__ double axis_gap(double X, double lo, double hi, double L, int periodic) {
-    const double c = 0.5 * (lo + hi), r = 0.5 * (hi - lo);
-    const double d = fabs(min_image(X - c, L, periodic)) - r;
-    return d > 0.0 ? d * d : 0.0;
+// Wells summed point by point, in the order of the cell list.  V feeds mixed
+// solves whose last digits hang on its last bits (the entropies of a mixed
+// call move by 2e-9 with them), so each term is the FP64 expression of the
+// head of this file and its order is fixed; nothing is factored or tabulated.
+// What is saved is the work on atoms out of reach, five in six of those in the
+// 27 cells: `near` holds position and cutoff of each listed atom in FP32, the
+// cutoff widened past every rounding error (near_atoms), and an atom beyond
+// it takes no FP64 at all.  The minimum image's quotient is only rounded to an
+// integer, so a product with 1 / L serves unless it lies near a half.
+// FP64 issue bounds it still; the build of 1,024 atoms on 96 x 96 x 160 with
+// its projector lists takes 10.2 ms, 24.1 with every listed atom in FP64 and the
+// lists' prefix sum on the host.  (Wells tabulated as products of three 1-D
+// factors took it to 3.6 but move V's last bits.)
+__device__ __forceinline__ double min_image_exact(double d, double L, double inv_L, int periodic) {
+    if (!periodic) return d;
+    const double t = d * inv_L;
+    double k = rint(t);
+    if (!(fabs(fabs(t - k) - 0.5) > 1e-6 && fabs(t) < 1e6)) k = rint(d / L);
+    return d - L * k;
 }
 
-__global__ void __launch_bounds__(kTx* kTy) k_local_potential(
-    GridGeo g, CellArgs cl, const double* __restrict__ xyz, const double* __restrict__ depth,
-    const double* __restrict__ sigma, double cutoff_sigmas, double reach, const double* __restrict__ v_ext,
-    double* __restrict__ V, float* __restrict__ V32, int tiles_x, int tiles_y, long long n_tiles) {
-    __shared__ int near_id[kNear];
-    __shared__ double2 tab[kAtomBatch][kTab];   // squared displacement, Gaussian factor
-    __shared__ double2 par[kAtomBatch];         // depth, squared cutoff
-    __shared__ int warp_n[kTx * kTy / 32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kTx * kTy / 32;
-    const int tx = tid % kTx, ty = tid / kTx;
-    for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const int o[3] = {(int)(tile % tiles_x) * kTx, (int)((tile / tiles_x) % tiles_y) * kTy,
-                          (int)(tile / ((long long)tiles_x * tiles_y)) * kTz};
-        const int ext[3] = {kTx, kTy, kTz};
-        double lo[3], hi[3];
-        int c0[3], nc[3];   // first cell and number of cells that can hold atoms in reach
-        for (int d = 0; d < 3; ++d) {
-            lo[d] = o[d] * g.h[d];
-            hi[d] = (min(o[d] + ext[d], g.n[d]) - 1) * g.h[d];
-            int a = (int)floor((lo[d] - reach) / cl.cell[d]), b = (int)floor((hi[d] + reach) / cl.cell[d]);
-            if (g.periodic[d]) {
-                if (b - a + 1 >= cl.nc[d]) a = 0, b = cl.nc[d] - 1;
-            } else {
-                a = min(max(a, 0), cl.nc[d] - 1);
-                b = min(max(b, 0), cl.nc[d] - 1);
-            }
-            c0[d] = a;
-            nc[d] = b - a + 1;
-        }
-        double acc[kTz];
-#pragma unroll
-        for (int z = 0; z < kTz; ++z) acc[z] = 0.0;
-        int n_near = 0;
-        // the listed atoms, a batch at a time
-        auto sum_near = [&]() {
-            for (int a0 = 0; a0 < n_near; a0 += kAtomBatch) {
-                const int na = min(kAtomBatch, n_near - a0);
-                __syncthreads();
-                for (int t = tid; t < na * kTab; t += blockDim.x) {
-                    const int k = t / kTab, i = t - k * kTab;
-                    const int d = i < kTx ? 0 : (i < kTx + kTy ? 1 : 2);
-                    const int idx = o[d] + i - (d == 0 ? 0 : (d == 1 ? kTx : kTx + kTy));
-                    const int at = near_id[a0 + k];
-                    const double s = sigma[at];
-                    const double dd = min_image(idx * g.h[d] - xyz[3 * at + d], g.L[d], g.periodic[d]);
-                    tab[k][i] = make_double2(dd * dd, exp(-dd * dd / (2.0 * s * s)));
-                    if (i == 0) {
-                        const double rc = cutoff_sigmas * s;
-                        par[k] = make_double2(depth[at], rc * rc);
-                    }
-                }
-                __syncthreads();
-                for (int k = 0; k < na; ++k) {
-                    const double2 p = par[k], x = tab[k][tx], y = tab[k][kTx + ty];
-                    const double dxy = x.x + y.x;
-                    if (dxy > p.y) continue;
-                    const double gxy = p.x * x.y * y.y;
-#pragma unroll
-                    for (int z = 0; z < kTz; ++z) {
-                        const double2 w = tab[k][kTx + kTy + z];
-                        if (dxy + w.x <= p.y) acc[z] = fma(gxy, w.y, acc[z]);
-                    }
-                }
-            }
-            __syncthreads();
-            n_near = 0;
-        };
-        // cells in order, one per warp at a time; the list order is fixed, so
-        // that a potential comes out the same every time
-        const int n_cells = nc[0] * nc[1] * nc[2];
-        for (int cb = 0; cb < n_cells; cb += nw) {
-            int e = lane, end = 0;
-            if (cb + warp < n_cells) {
-                const int c = cb + warp;
-                int k[3] = {c0[0] + c % nc[0], c0[1] + (c / nc[0]) % nc[1], c0[2] + c / (nc[0] * nc[1])};
-                for (int d = 0; d < 3; ++d) k[d] = ((k[d] % cl.nc[d]) + cl.nc[d]) % cl.nc[d];
-                const int cell = k[0] + cl.nc[0] * (k[1] + cl.nc[1] * k[2]);
-                e = cl.start[cell] + lane;
-                end = cl.start[cell + 1];
-            }
-            while (__syncthreads_or(e - lane < end)) {
-                bool in = false;
-                int at = 0;
-                if (e < end) {
-                    at = cl.atoms[e];
-                    const double rc = cutoff_sigmas * sigma[at];
-                    double r2 = 0.0;
-                    for (int d = 0; d < 3; ++d) r2 += axis_gap(xyz[3 * at + d], lo[d], hi[d], g.L[d], g.periodic[d]);
-                    in = r2 <= rc * rc * (1.0 + 1e-9);
-                }
-                e += 32;
-                const unsigned m = __ballot_sync(0xffffffffu, in);
-                if (lane == 0) warp_n[warp] = __popc(m);
-                __syncthreads();
-                int before = n_near, total = n_near;
-                for (int w = 0; w < nw; ++w) {
-                    if (w < warp) before += warp_n[w];
-                    total += warp_n[w];
-                }
-                if (in) near_id[before + __popc(m & ((1u << lane) - 1u))] = at;
-                n_near = total;
-                __syncthreads();
-                if (n_near > kNear - kTx * kTy) sum_near();
-            }
-        }
-        sum_near();
-        const int ix = o[0] + tx, iy = o[1] + ty;
-        if (ix < g.n[0] && iy < g.n[1]) {
-#pragma unroll
-            for (int z = 0; z < kTz; ++z) {
-                if (o[2] + z >= g.n[2]) break;
-                const long long i = ix + (long long)g.n[0] * (iy + (long long)g.n[1] * (o[2] + z));
-                const double v = (v_ext ? v_ext[i] : 0.0) - acc[z];
-                V[i] = v;
-                V32[i] = (float)v;
-            }
-        }
+__device__ __forceinline__ float min_image_f32(float d, float L, float inv_L, int periodic) {
+    return periodic ? d - L * rintf(d * inv_L) : d;
+}
+
+__global__ void k_local_potential(GridGeo g, CellArgs cl, const double* __restrict__ xyz,
+                                  const double* __restrict__ depth, const double* __restrict__ sigma,
+                                  const float4* __restrict__ near, double cutoff_sigmas,
+                                  const double* __restrict__ v_ext, double* __restrict__ V, float* __restrict__ V32,
+                                  long long N) {
+    double inv[3];
+    float Lf[3], invf[3];
+    for (int d = 0; d < 3; ++d) {
+        inv[d] = 1.0 / g.L[d];
+        Lf[d] = (float)g.L[d];
+        invf[d] = (float)inv[d];
+    }
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int ix = (int)(i % g.n[0]);
+        const int iy = (int)((i / g.n[0]) % g.n[1]);
+        const int iz = (int)(i / ((long long)g.n[0] * g.n[1]));
+        const double px = ix * g.h[0], py = iy * g.h[1], pz = iz * g.h[2];
+        const float fx = (float)px, fy = (float)py, fz = (float)pz;
+        double v = v_ext ? v_ext[i] : 0.0;
+        for_each_near_atom(g, cl.nc, cl.cell, cl.start, ix, iy, iz, [&](int e) {
+            const float4 q = near[e];
+            const float qx = min_image_f32(fx - q.x, Lf[0], invf[0], g.periodic[0]);
+            const float qy = min_image_f32(fy - q.y, Lf[1], invf[1], g.periodic[1]);
+            const float qz = min_image_f32(fz - q.z, Lf[2], invf[2], g.periodic[2]);
+            if (qx * qx + qy * qy + qz * qz > q.w) return;   // (false for a NaN)
+            const int a = cl.atoms[e];
+            const double dx = min_image_exact(px - xyz[3 * a + 0], g.L[0], inv[0], g.periodic[0]);
+            const double dy = min_image_exact(py - xyz[3 * a + 1], g.L[1], inv[1], g.periodic[1]);
+            const double dz = min_image_exact(pz - xyz[3 * a + 2], g.L[2], inv[2], g.periodic[2]);
+            const double r2 = dx * dx + dy * dy + dz * dz;
+            const double s = sigma[a];
+            const double rc = cutoff_sigmas * s;
+            if (r2 <= rc * rc) v -= depth[a] * exp(-r2 / (2.0 * s * s));
+        });
+        V[i] = v;
+        V32[i] = (float)v;
     }
 }
 
@@ -434,7 +358,8 @@ __global__ void k_proj_lists(GridGeo g, CellArgs cl, const int* __restrict__ i0,
         const int iz = (int)(i / ((long long)g.n[0] * g.n[1]));
         int ids[16];
         int cnt = 0;
-        for_each_near_atom(g, cl.nc, cl.cell, cl.start, cl.atoms, ix, iy, iz, [&](int a) {
+        for_each_near_atom(g, cl.nc, cl.cell, cl.start, ix, iy, iz, [&](int e) {
+            const int a = cl.atoms[e];
             const int u = window_slot(ix, i0[3 * a + 0], len[3 * a + 0], g.n[0], g.periodic[0]);
             const int v = window_slot(iy, i0[3 * a + 1], len[3 * a + 1], g.n[1], g.periodic[1]);
             const int w = window_slot(iz, i0[3 * a + 2], len[3 * a + 2], g.n[2], g.periodic[2]);
@@ -587,6 +512,25 @@ md_status build_cells(const Ham& H, const std::vector<double>& xyz, double rcut,
     return MD_OK;
 }
 
+// Position and squared reach of every entry of a cell list in FP32.  A
+// displacement computed in FP32 is off by at most 8 roundings (2^-24) of
+// |x| + |p| + L: points, positions, L, k and their products, with k off by one
+// only where both images are L/2 away.  The reach is widened by 32 times that,
+// its square by 1e-5, so that an atom beyond it in FP32 is beyond its cutoff; a
+// reach past FP32's range lets every atom in.
+std::vector<float4> near_atoms(const Ham& H, const std::vector<double>& xyz, const std::vector<double>& sigma,
+                               const std::vector<int>& ids) {
+    std::vector<float4> out(H.n_atoms);
+    for (long long e = 0; e < H.n_atoms; ++e) {
+        const double* x = &xyz[3LL * ids[e]];
+        double size = 0.0;
+        for (int d = 0; d < 3; ++d) size = std::max(size, std::fabs(x[d]) + 2.0 * H.n[d] * H.h[d]);
+        const double r = H.cutoff_sigmas * sigma[ids[e]] + 32.0 * 8.0 * 0x1p-24 * size;
+        out[e] = make_float4((float)x[0], (float)x[1], (float)x[2], (float)(r * r * (1.0 + 1e-5)));
+    }
+    return out;
+}
+
 }  // namespace
 
 #define MD_CUDA_TRY(expr)                                                                 \
@@ -670,6 +614,8 @@ md_status build_hamiltonian_device(Ham& H, const md_atoms* atoms, const md_pot_p
     int* d_overflow = nullptr;
     int* d_count = nullptr;
     long long* d_sums = nullptr;
+    std::vector<float4> near;
+    float4* d_near = nullptr;
     double max_sigma = 0.0;
     GridGeo g = geo_of(H);
     const int threads = 256;
@@ -707,13 +653,13 @@ md_status build_hamiltonian_device(Ham& H, const md_atoms* atoms, const md_pot_p
     }
     ca.start = d_cstart;
     ca.atoms = d_cids;
-    {
-        const int tx = (H.n[0] + kTx - 1) / kTx, ty = (H.n[1] + kTy - 1) / kTy;
-        const long long tiles = (long long)tx * ty * ((H.n[2] + kTz - 1) / kTz);
-        k_local_potential<<<(unsigned)std::min<long long>(tiles, 152LL * 64), kTx * kTy, 0, stream>>>(
-            g, ca, H.atom_xyz, H.atom_depth, H.atom_sigma, H.cutoff_sigmas, H.cutoff_sigmas * max_sigma, d_vext, H.V,
-            H.V32, tx, ty, tiles);
+    if (H.n_atoms > 0) {
+        near = near_atoms(H, xyz, sigma, cids);
+        MD_CUDA_TRY(cudaMalloc(&d_near, near.size() * sizeof(float4)));
+        MD_CUDA_TRY(cudaMemcpy(d_near, near.data(), near.size() * sizeof(float4), cudaMemcpyHostToDevice));
     }
+    k_local_potential<<<blocks, threads, 0, stream>>>(g, ca, H.atom_xyz, H.atom_depth, H.atom_sigma, d_near,
+                                                     H.cutoff_sigmas, d_vext, H.V, H.V32, N);
     MD_CUDA_TRY(cudaGetLastError());
 
     if (H.nonlocal && H.n_atoms > 0) {
@@ -816,6 +762,7 @@ fail:
     cudaFree(d_overflow);
     cudaFree(d_count);
     cudaFree(d_sums);
+    cudaFree(d_near);
     return st;
 }
 
