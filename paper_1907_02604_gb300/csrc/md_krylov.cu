@@ -196,7 +196,10 @@ struct KChunk {      // up to kKryChunkRows rows of one atom
 
 struct KShared {
     long long part[kMaxWarps][4];
-    long long mbox[kMaxC][7];     // per rank: u.w (2), w.w (2), stop flag of rank 0, ||w - alpha u||^2 (2)
+    // per rank: u.w (2), w.w (2), stop flag of rank 0, ||w - alpha u||^2 (2), defect
+    // of the FP64 check (a word of its own: no barrier of the cluster lies between
+    // rank 0's reads of the last step's words and the check of a CTA with little to do)
+    long long mbox[kMaxC][8];
     int2 ca, cg;                  // alpha and g as limbs
     int e;                        // u_new = (w - alpha u) 2^e
     int zlo[kMaxC + 1];           // first plane of each rank's slab
@@ -1273,10 +1276,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
             if (tid == 0) {
                 s2 = 0.0;
                 for (int k = 0; k <= nwp; ++k) s2 += __longlong_as_double(S.part[k][0]);
-                k_st_remote(k_map(smem_addr(&S.mbox[rank][0]), 0), __double_as_longlong(s2));
+                k_st_remote(k_map(smem_addr(&S.mbox[rank][7]), 0), __double_as_longlong(s2));
             }
             k_sync();
-            for (int r = 0; r < C; ++r) defect += __longlong_as_double(S.mbox[r][0]);
+            for (int r = 0; r < C; ++r) defect += __longlong_as_double(S.mbox[r][7]);   // rank 0 holds them
             defect = sqrt(defect * S.inv0) * P.scale;   // relative to ||u||, in units of H
         }
         // ---- outputs of the solution vectors ----------------------------------
