@@ -283,6 +283,7 @@ void kry_operator(KrylovParams& P, const Ham& H, double scale) {
             const long long x = o < H.q ? std::llrint(std::ldexp(H.coef[d][o] / scale, 62)) : 0;
             const long long hi = (x + (1LL << 30)) >> 31;
             P.wh[d][o] = (int)hi;
+            P.wl[d][o] = (int)(x - (hi << 31));
             const float f[2] = {(float)(x - (hi << 31)), (float)hi};
             std::memcpy(&P.wf[d][o], f, sizeof(f));
         }

@@ -19,9 +19,10 @@
 // FP64 FMAs per clock and SM against 31 integer multiply-adds into 64 bits
 // and 115 FP32 FMAs (measured).  So the vectors are 62-bit fixed point: a
 // value u is hi 2^-31 + lo 2^-62 with two signed 31-bit limbs.  Of a product,
-// hi hi is exact in a 64-bit integer sum and the mixed terms, 2^-31 of it,
-// are FP32 (2^-55 of the product); the lo lo term, below 2^-62, is dropped,
-// except in w.w, where it adds up.  Each result is rounded once to 2^-62.
+// hi hi is exact in a 64-bit integer sum; the mixed terms, 2^-31 of it, are
+// 64-bit integers in FP64 calls and FP32 in mixed precision; the lo lo term,
+// below 2^-62, is dropped, except in w.w, where it adds up.  Each result is
+// rounded once to 2^-62.
 // Vectors are kept at norm [1/8, 1/4) by exact powers of two, so the rounding
 // is ~1e-16 of the norm per step, the size of FP64's.  A = (H_R - shift) /
 // scale has ||A|| < 1/2, which bounds every sum below the 64-bit range.
@@ -47,7 +48,8 @@
 // registers): 255 instructions a point-step without projectors, 560 with
 // them, at 1.9 and 1.7 issued a clock.  96 nodes x 16 poles on 33^3 regions
 // with projectors take 108 ms, 506 with one complex COCG per pole in mixed
-// precision; 13 nodes x 16 poles on 25^3 in FP64 9.1 ms against 278.
+// precision; 13 nodes x 16 poles on 25^3 in FP64 8.6 ms against 278 (9.1 with
+// FP32 mixed terms).
 #include <cuda_runtime.h>
 
 #include <cfloat>
@@ -116,10 +118,17 @@ __device__ __forceinline__ int2 split31(long long x) {
     return make_int2(opaque((int)(x >> 31)), opaque((int)(x & 0x7fffffffLL) - (1 << 30)));
 }
 // A product of two 62-bit values is hi hi 2^-62 + (hi lo + lo hi) 2^-93 + ..:
-// the first term exactly, in 64 bits; the mixed terms, 2^-31 of it, in FP32
-// (2^-55 of the product, FP64's own rounding is 2^-54).  IMAD.WIDE with
-// distinct operands runs at 31 a clock and SM (measured), FFMA2 at 65 pairs,
-// so the mixed terms cost a quarter of what they did in 64-bit integers.
+// the first term exactly, in 64 bits; the mixed terms, 2^-31 of it, in one of
+// two ways.
+// Mixed precision (X = false): in FP32.  IMAD.WIDE with distinct operands runs
+// at 31 a clock and SM (measured), FFMA2 at 65 pairs, so they cost a quarter of
+// what they do in integers.  But lo is as large where hi is small, and 24 bits
+// of lo hi leave 2^-57 on every component: against 64-bit Jacobi matrices,
+// beta is off by 5e-15 after a few steps and alpha by 1e-13 after 40 on 17^3
+// regions.
+// FP64 calls (X = true): in 64-bit integers, exact but for the terms' last 8
+// bits; beta is within 1e-15 and alpha within 5e-15 there (FP64 arithmetic:
+// 1e-15 and 1e-14).
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 pack(float a, float b) {
     f32x2 r;
@@ -135,58 +144,172 @@ __device__ __forceinline__ float sum2(f32x2 v) {
 __device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
+__device__ __forceinline__ float as_float(int x) { return __int_as_float(x); }
+__device__ __forceinline__ int as_int(float x) { return __float_as_int(x); }
+// Left operand: {(float)hi, (float)lo} or lo beside hi; right operand the same
+// with {(float)lo, (float)hi}.
+template <bool X>
+struct Lhs {
+    int h;
+    f32x2 f;
+    __device__ __forceinline__ Lhs(int hi, int lo) : h(hi), f(pack((float)hi, (float)lo)) {}
+};
+template <>
+struct Lhs<true> {
+    int h, l;
+    __device__ __forceinline__ Lhs(int hi, int lo) : h(hi), l(lo) {}
+};
+template <bool X>
+struct Rhs {
+    int h;
+    f32x2 f;
+    __device__ __forceinline__ Rhs(int hi, int lo) : h(hi), f(pack((float)lo, (float)hi)) {}
+    __device__ __forceinline__ Rhs(int hi, int, f32x2 lo_hi) : h(hi), f(lo_hi) {}
+};
+template <>
+struct Rhs<true> {
+    int h, l;
+    __device__ __forceinline__ Rhs(int hi, int lo) : h(hi), l(lo) {}
+    __device__ __forceinline__ Rhs(int hi, int lo, f32x2) : h(hi), l(lo) {}
+};
+// A table entry: (hi, bits of (float)lo), or (hi, lo).  A pair of floats in
+// registers would have to be assembled by moves, so its mixed terms are single
+// FMAs.
+template <bool X>
+struct TabVal {
+    int h;
+    float f, l;
+    __device__ __forceinline__ TabVal(int hi, int lo) : h(hi), f((float)hi), l(as_float(lo)) {}
+};
+template <>
+struct TabVal<true> {
+    int h, l;
+    __device__ __forceinline__ TabVal(int hi, int lo) : h(hi), l(lo) {}
+};
+template <bool X>
+__device__ __forceinline__ int2 tab_limbs(int2 v) {
+    return X ? v : make_int2(v.x, as_int((float)v.y));
+}
+template <bool X>
+__device__ __forceinline__ int4 tab_entry(int4 v) {
+    const int2 a = tab_limbs<X>(make_int2(v.x, v.y)), b = tab_limbs<X>(make_int2(v.z, v.w));
+    return make_int4(a.x, a.y, b.x, b.y);
+}
+// a value from its limbs
+template <bool X>
+__device__ __forceinline__ TabVal<X> tab_of(int2 v) {
+    const int2 t = tab_limbs<X>(make_int2(opaque(v.x), X ? opaque(v.y) : v.y));
+    return TabVal<X>(t.x, t.y);
+}
+template <bool X>
 struct Acc {
     long long hh = 0;
     f32x2 f = 0;      // mixed terms, units of 2^-93
     float s = 0.f;    // those of table entries
-    // += (ah, af) * (bh, bf), af = {(float)hi, (float)lo}, bf = {(float)lo, (float)hi}
-    __device__ __forceinline__ void mac(int ah, f32x2 af, int bh, f32x2 bf) {
-        madw(hh, ah, bh);
-        fma2(f, af, bf);
+    __device__ __forceinline__ void mac(const Lhs<X>& a, const Rhs<X>& b) {
+        madw(hh, a.h, b.h);
+        fma2(f, a.f, b.f);
     }
-    // += (ah, (float)ah, al) * (bh, (float)bh, bl)
-    __device__ __forceinline__ void mac(int ah, float af, float al, int bh, float bf, float bl) {
-        madw(hh, ah, bh);
-        s = fmaf(af, bl, fmaf(al, bf, s));
+    __device__ __forceinline__ void mac(const TabVal<X>& a, const TabVal<X>& b) {
+        madw(hh, a.h, b.h);
+        s = fmaf(a.f, b.l, fmaf(a.l, b.f, s));
+    }
+    // a b + c d of one projector row
+    __device__ __forceinline__ void mac(const TabVal<X>& a, const TabVal<X>& b, const TabVal<X>& c, const TabVal<X>& d) {
+        mac(a, b);
+        mac(c, d);
     }
     // rounded to 2^-62; |mixed| < 2^62, as ||u|| < 1/4
     __device__ __forceinline__ long long fold() const { return hh + __float2int_rn((sum2(f) + s) * 0x1p-31f); }
 };
-__device__ __forceinline__ f32x2 hi_lo(int h, int l) { return pack((float)h, (float)l); }
-__device__ __forceinline__ f32x2 lo_hi(int h, int l) { return pack((float)l, (float)h); }
-// A table entry (hi, bits of (float)lo) as operand; a pair in registers would
-// have to be assembled by moves, so these mixed terms are single FMAs.
-struct TabVal {
-    int h;
-    float f, l;
+template <>
+struct Acc<true> {
+    long long hh = 0;
+    // Mixed terms, units of 2^-93, and those of projector rows, units of 2^-85.
+    // |hi lo| sums to less than 2^61.9 over the stencil (the |u| of 27 points of a
+    // vector of norm 1/4: 1.75), |lo hi| to 2^62 (weights: 2^30, V and g: 2^31.6).
+    long long hl = 0, lh = 0, hs = 0;
+    __device__ __forceinline__ void mac(const Lhs<true>& a, const Rhs<true>& b) {
+        madw(hh, a.h, b.h);
+        madw(hl, a.h, b.l);
+        madw(lh, a.l, b.h);
+    }
+    __device__ __forceinline__ void mac(const TabVal<true>& a, const TabVal<true>& b) {
+        madw(hh, a.h, b.h);
+        madw(hl, a.h, b.l);
+        madw(lh, a.l, b.h);
+    }
+    // (up to 16 rows meet at a point: a row's mixed terms, below 2^62.7, are
+    // scaled before they are added)
+    __device__ __forceinline__ void mac(const TabVal<true>& a, const TabVal<true>& b, const TabVal<true>& c,
+                                        const TabVal<true>& d) {
+        madw(hh, a.h, b.h);
+        madw(hh, c.h, d.h);
+        long long m = 0;
+        madw(m, a.h, b.l);
+        madw(m, a.l, b.h);
+        madw(m, c.h, d.l);
+        madw(m, c.l, d.h);
+        hs += m >> 8;
+    }
+    __device__ __forceinline__ long long fold() const { return hh + ((((hl + lh) >> 8) + hs + (1LL << 22)) >> 23); }
 };
-__device__ __forceinline__ TabVal tv(int hi, int lo) { return TabVal{hi, (float)hi, __int_as_float(lo)}; }
-__device__ __forceinline__ void tmac(Acc& a, const TabVal& x, const TabVal& y) { a.mac(x.h, x.f, x.l, y.h, y.f, y.l); }
-__device__ __forceinline__ int2 tab_limbs(int2 v) { return make_int2(v.x, __float_as_int((float)v.y)); }
-// Partial sums of u.w and w.w: hi hi exact, the rest in float (lo lo terms
-// included: in w.w they add up, 2e-13 of the sum).
+// Partial sums of u.w and w.w: hi hi exact, the mixed terms in float or, 16
+// points at a time, in integers; the lo lo terms (in w.w they add up, 2e-13 of
+// the sum) in float.
+template <bool X>
 struct Dots {
     long long hh1 = 0, hh2 = 0;
     f32x2 f1 = 0, f2 = 0;
     float q1 = 0.f;
-    __device__ __forceinline__ void add(int uh, f32x2 uf, int2 w) {
-        madw(hh1, uh, w.x);
+    __device__ __forceinline__ void add(const Lhs<X>& u, int2 w) {
+        madw(hh1, u.h, w.x);
         madw(hh2, w.x, w.x);
         const float wh = (float)w.x, wl = (float)w.y;
-        fma2(f1, uf, pack(wl, wh));
+        fma2(f1, u.f, pack(wl, wh));
         fma2(f2, pack(wh, wl), pack(wl, wl * 0x1p-32f));
-        q1 = fmaf(__uint_as_float((uint32_t)(uf >> 32)), wl * 0x1p-31f, q1);
+        q1 = fmaf(__uint_as_float((uint32_t)(u.f >> 32)), wl * 0x1p-31f, q1);
     }
+    __device__ __forceinline__ void flush() {}
     // mixed parts in units of 2^-83 (w.w: half of them)
     __device__ __forceinline__ long long l1() const { return __float2ll_rn((sum2(f1) + q1) * 0x1p-10f); }
     __device__ __forceinline__ long long l2() const { return __float2ll_rn(sum2(f2) * 0x1p-10f); }
+};
+template <>
+struct Dots<true> {
+    long long hh1 = 0, hh2 = 0;
+    long long x1 = 0, y1 = 0, x2 = 0, s1 = 0, s2 = 0;
+    float q1 = 0.f, q2 = 0.f;
+    int n = 0;
+    __device__ __forceinline__ void add(const Lhs<true>& u, int2 w) {
+        madw(hh1, u.h, w.x);
+        madw(x1, u.h, w.y);
+        madw(y1, u.l, w.x);
+        madw(hh2, w.x, w.x);
+        madw(x2, w.x, w.y);
+        const float f = (float)w.y;
+        q1 = fmaf((float)u.l, f, q1);
+        q2 = fmaf(f, f, q2);
+    }
+    // after every pair: 8 pairs of |hi| <= 2^29 times |lo| <= 2^30 stay below 2^63
+    __device__ __forceinline__ void flush() {
+        if ((++n & 7) == 0) {
+            s1 += (x1 >> 10) + (y1 >> 10);
+            s2 += x2 >> 10;
+            x1 = y1 = x2 = 0;
+        }
+    }
+    __device__ __forceinline__ long long l1() const {
+        return s1 + (x1 >> 10) + (y1 >> 10) + __float2ll_rn(q1 * 0x1p-41f);
+    }
+    __device__ __forceinline__ long long l2() const { return s2 + (x2 >> 10) + __float2ll_rn(q2 * 0x1p-42f); }
 };
 __device__ __forceinline__ int2 to_limbs(double v) { return split31(__double2ll_rn(v * 0x1p62)); }
 
 struct KRow {        // one run of a projector row inside the slab
     int voff;        // index of window slot 0 in the u buffer
     int uu;          // u0 | u1 << 8 | local atom << 16
-    int2 r0, r1, r2; // g_y g_z, (d g)_y g_z, g_y (d g)_z: hi, (float)lo
+    int2 r0, r1, r2; // g_y g_z, (d g)_y g_z, g_y (d g)_z: hi, lo (a float in mixed precision)
 };
 static_assert(sizeof(KRow) == 32, "row record");
 
@@ -244,6 +367,7 @@ __device__ __forceinline__ int slab_lo(int m2, int C, int r) { return r * (m2 / 
 // of points (2k, 2k+1) of a region row the projector rows that cover one or
 // both: 1 + row id | x table entry of the first << 16, entry of the second
 // (entry and row 0 are zeros: a point outside the row, an empty record).
+template <bool X>
 __device__ void build_rows(const KrylovParams& P, const int m[3], const int lo[3], int z0, int depth, int q,
                            int pitch, int pp, KSharedNl& S, KRow* rows, KChunk* chunks, int4* xtab, int* cnt,
                            uint2* rec) {
@@ -318,14 +442,14 @@ __device__ void build_rows(const KrylovParams& P, const int m[3], const int lo[3
                     const int sh = rx.shift[run];
                     r.voff = (c - z0 + q) * pp + b * pitch + sh;
                     r.uu = u0 | (u1 << 8) | (k << 16);
-                    const int4 y = ty[vv], z = tz[ww];
-                    Acc r0, r1, r2;
-                    tmac(r0, tv(y.x, y.y), tv(z.x, z.y));
-                    tmac(r1, tv(y.z, y.w), tv(z.x, z.y));
-                    tmac(r2, tv(y.x, y.y), tv(z.z, z.w));
-                    r.r0 = tab_limbs(split31(r0.fold()));
-                    r.r1 = tab_limbs(split31(r1.fold()));
-                    r.r2 = tab_limbs(split31(r2.fold()));
+                    const int4 y = tab_entry<X>(ty[vv]), z = tab_entry<X>(tz[ww]);
+                    Acc<X> r0, r1, r2;
+                    r0.mac(TabVal<X>(y.x, y.y), TabVal<X>(z.x, z.y));
+                    r1.mac(TabVal<X>(y.z, y.w), TabVal<X>(z.x, z.y));
+                    r2.mac(TabVal<X>(y.x, y.y), TabVal<X>(z.z, z.w));
+                    r.r0 = tab_limbs<X>(split31(r0.fold()));
+                    r.r1 = tab_limbs<X>(split31(r1.fold()));
+                    r.r2 = tab_limbs<X>(split31(r2.fold()));
                     rows[id] = r;
                     const int item0 = ((c - z0) * m[1] + b) * npx;
                     for (int pr = (u0 + sh) >> 1; pr <= (u1 + sh) >> 1; ++pr) {
@@ -360,7 +484,7 @@ __device__ void build_rows(const KrylovParams& P, const int m[3], const int lo[3
                 for (int i = lane; i < nch; i += 32)
                     chunks[cf + i] = KChunk{first + kKryChunkRows * i, min(kKryChunkRows, total - kKryChunkRows * i), k,
                                             1 + tab * P.win_x};
-                for (int u = lane; u < P.win_x; u += 32) xtab[1 + tab * P.win_x + u] = tx[u];
+                for (int u = lane; u < P.win_x; u += 32) xtab[1 + tab * P.win_x + u] = tab_entry<X>(tx[u]);
             }
         }
     }
@@ -387,6 +511,7 @@ __device__ __forceinline__ long long warp_sum4(long long s0, long long s1, long 
 // the row's three y z factors R; the x tables enter once, at the end.
 // (A lane per row, each walking its run with both x tables, took 21,800
 // cycles a step on the bulk regions, four times the issue slots.)
+template <bool X>
 __device__ __forceinline__ void project(const KrylovParams& P, const int2* __restrict__ U, const KRow* rows,
                                         const KChunk* chunks, int n_chunks, int nw, const int4* xtab, int4* stage,
                                         long long* acc) {
@@ -415,7 +540,7 @@ __device__ __forceinline__ void project(const KrylovParams& P, const int2* __res
         long long s0 = 0, s1 = 0, s2 = 0, s3 = 0;
         for (int ub = 0; ub < P.win_x; ub += 16) {
             const int u = ub + (lane & 15);
-            Acc A0, A1, A2;
+            Acc<X> A0, A1, A2;
             const int4* st = stage + 2 * half;
             // rows past the count are empty runs, so the half warps stay together
 #pragma unroll 4
@@ -424,21 +549,20 @@ __device__ __forceinline__ void project(const KrylovParams& P, const int2* __res
                 const int u0 = a.y & 0xff, u1 = (a.y >> 8) & 0xff;
                 int2 v = make_int2(0, 0);
                 if (u >= u0 && u <= u1) v = U[a.x + u];
-                v.x = opaque(v.x);
-                const float vh = (float)v.x, vl = (float)v.y;
-                A0.mac(v.x, vh, vl, a.z, (float)a.z, __int_as_float(a.w));
-                A1.mac(v.x, vh, vl, b.x, (float)b.x, __int_as_float(b.y));
-                A2.mac(v.x, vh, vl, b.z, (float)b.z, __int_as_float(b.w));
+                const TabVal<X> t = tab_of<X>(v);
+                A0.mac(t, TabVal<X>(a.z, a.w));
+                A1.mac(t, TabVal<X>(b.x, b.y));
+                A2.mac(t, TabVal<X>(b.z, b.w));
             }
             const int4 t = u < P.win_x ? xtab[k.tab + u] : make_int4(0, 0, 0, 0);
-            const TabVal g = tv(t.x, t.y), dg = tv(t.z, t.w);
-            const int2 l0 = tab_limbs(split31(A0.fold())), l1 = tab_limbs(split31(A1.fold()));
-            const int2 l2 = tab_limbs(split31(A2.fold()));
-            Acc r0, r1, r2, r3;
-            tmac(r0, tv(l0.x, l0.y), g);
-            tmac(r1, tv(l0.x, l0.y), dg);
-            tmac(r2, tv(l1.x, l1.y), g);
-            tmac(r3, tv(l2.x, l2.y), g);
+            const TabVal<X> g(t.x, t.y), dg(t.z, t.w);
+            const int2 l0 = tab_limbs<X>(split31(A0.fold())), l1 = tab_limbs<X>(split31(A1.fold()));
+            const int2 l2 = tab_limbs<X>(split31(A2.fold()));
+            Acc<X> r0, r1, r2, r3;
+            r0.mac(TabVal<X>(l0.x, l0.y), g);
+            r1.mac(TabVal<X>(l0.x, l0.y), dg);
+            r2.mac(TabVal<X>(l1.x, l1.y), g);
+            r3.mac(TabVal<X>(l2.x, l2.y), g);
             s0 += r0.fold();
             s1 += r1.fold();
             s2 += r2.fold();
@@ -452,16 +576,17 @@ __device__ __forceinline__ void project(const KrylovParams& P, const int2* __res
 
 // One row's factors of the apply: nonlocal(u)(i) = sum over the rows that
 // cover i of g_x K1 + (d g)_x K2.
+template <bool X>
 __device__ __forceinline__ int4 row_factors(const KRow* row, const int2* cl) {
     const int4 a = reinterpret_cast<const int4*>(row)[0], b = reinterpret_cast<const int4*>(row)[1];
     const int4* c = reinterpret_cast<const int4*>(cl + 4 * ((a.y >> 16) & 0xff));
     const int4 c01 = c[0], c23 = c[1];
-    Acc k1, k2;
-    tmac(k1, tv(a.z, a.w), tv(c01.x, c01.y));
-    tmac(k1, tv(b.x, b.y), tv(c23.x, c23.y));
-    tmac(k1, tv(b.z, b.w), tv(c23.z, c23.w));
-    tmac(k2, tv(a.z, a.w), tv(c01.z, c01.w));
-    const int2 x = tab_limbs(split31(k1.fold())), y = tab_limbs(split31(k2.fold()));
+    Acc<X> k1, k2;
+    k1.mac(TabVal<X>(a.z, a.w), TabVal<X>(c01.x, c01.y));
+    k1.mac(TabVal<X>(b.x, b.y), TabVal<X>(c23.x, c23.y));
+    k1.mac(TabVal<X>(b.z, b.w), TabVal<X>(c23.z, c23.w));
+    k2.mac(TabVal<X>(a.z, a.w), TabVal<X>(c01.z, c01.w));
+    const int2 x = tab_limbs<X>(split31(k1.fold())), y = tab_limbs<X>(split31(k2.fold()));
     return make_int4(x.x, x.y, y.x, y.y);
 }
 
@@ -478,23 +603,25 @@ struct SlabArgs {
 };
 
 // Nonlocal term of one record entry on both points of a pair.
-__device__ __forceinline__ void nl_entry(const int4* ktab, const int4* xtab, uint32_t e0, uint32_t e1, Acc (&acc)[2]) {
+template <bool X>
+__device__ __forceinline__ void nl_entry(const int4* ktab, const int4* xtab, uint32_t e0, uint32_t e1,
+                                         Acc<X> (&acc)[2]) {
     const int4 k = ktab[e0 & 0xffffu], t0 = xtab[e0 >> 16], t1 = xtab[e1];
-    const TabVal k1 = tv(k.x, k.y), k2 = tv(k.z, k.w);
-    tmac(acc[0], tv(t0.x, t0.y), k1);
-    tmac(acc[1], tv(t1.x, t1.y), k1);
-    tmac(acc[0], tv(t0.z, t0.w), k2);
-    tmac(acc[1], tv(t1.z, t1.w), k2);
+    const TabVal<X> k1(k.x, k.y), k2(k.z, k.w);
+    acc[0].mac(TabVal<X>(t0.x, t0.y), k1, TabVal<X>(t0.z, t0.w), k2);
+    acc[1].mac(TabVal<X>(t1.x, t1.y), k1, TabVal<X>(t1.z, t1.w), k2);
 }
 
 // Sums of the stencil's off-diagonal terms on a pair at p (16-byte units);
 // kInside: the rows b-Q .. b+Q all lie in the region.
-template <int Q, bool kInside>
+template <int Q, bool kInside, bool X>
 __device__ __forceinline__ void stencil(const KrylovParams& P, const SlabArgs& A, const int4* p, int4 c, int a, int b,
-                                        Acc (&acc)[2]) {
+                                        Acc<X> (&acc)[2]) {
     constexpr int H = (Q + 1) / 2;   // loads on either side of the pair
     const int pitch = A.pitch >> 1, pp = A.pp >> 1;
-    auto add = [&](int i, int h, int l, int d, int o) { acc[i].mac(h, hi_lo(h, l), P.wh[d][o - 1], P.wf[d][o - 1]); };
+    auto add = [&](int i, int h, int l, int d, int o) {
+        acc[i].mac(Lhs<X>(h, l), Rhs<X>(P.wh[d][o - 1], P.wl[d][o - 1], P.wf[d][o - 1]));
+    };
     {
         int2 x[2 * (2 * H + 1)];     // the row around the pair: x[2H], x[2H+1] are its points
 #pragma unroll
@@ -531,10 +658,10 @@ __device__ __forceinline__ void stencil(const KrylovParams& P, const SlabArgs& A
 // shared memory: a column's z values kept in registers along a march save
 // seven of the twenty 16-byte loads of a pair but need more than 128 registers,
 // and 19 warps at 96 registers are the faster trade.
-template <int Q, bool kNl>
+template <int Q, bool kNl, bool X>
 __device__ __forceinline__ void slab_apply(const KrylovParams& P, const SlabArgs& A, const int4* ktab,
-                                           const int4* xtab, const int4* u_prev, int nw, int2 g, Dots& dots) {
-    const f32x2 gf = lo_hi(g.x, g.y);
+                                           const int4* xtab, const int4* u_prev, int nw, int2 g, Dots<X>& dots) {
+    const Rhs<X> gr(opaque(g.x), opaque(g.y));
     // lanes past the last pair repeat it and add nothing, so that warps stay whole
     for (int i0 = threadIdx.x & ~31; i0 < A.n_items; i0 += 32 * nw) {
         const int i = i0 + (int)(threadIdx.x & 31);
@@ -547,15 +674,14 @@ __device__ __forceinline__ void slab_apply(const KrylovParams& P, const SlabArgs
         const int b = (int)fdiv((uint32_t)pc, A.div_px), a = 2 * (pc - b * A.npx);
         const int4* p = reinterpret_cast<const int4*>(A.U + (d + Q) * A.pp + b * A.pitch + a);
         const int4 c = *p;
-        Acc acc[2];
+        Acc<X> acc[2];
         if (__all_sync(0xffffffffu, b >= Q && b + Q < A.m1)) stencil<Q, true>(P, A, p, c, a, b, acc);
         else stencil<Q, false>(P, A, p, c, a, b, acc);
-        const f32x2 c0 = hi_lo(c.x, c.y), c1 = hi_lo(c.z, c.w);
-        acc[0].mac(c.x, c0, v.x, lo_hi(v.x, v.y));
-        acc[1].mac(c.z, c1, v.z, lo_hi(v.z, v.w));
-        const int gx = opaque(g.x);
-        acc[0].mac(um.x, hi_lo(um.x, um.y), gx, gf);
-        acc[1].mac(um.z, hi_lo(um.z, um.w), gx, gf);
+        const Lhs<X> c0(c.x, c.y), c1(c.z, c.w);
+        acc[0].mac(c0, Rhs<X>(v.x, v.y));
+        acc[1].mac(c1, Rhs<X>(v.z, v.w));
+        acc[0].mac(Lhs<X>(um.x, um.y), gr);
+        acc[1].mac(Lhs<X>(um.z, um.w), gr);
         if constexpr (kNl) {
             for (int q = 0; q < P.rec_words; ++q) {
                 const uint4 r = q == 0 ? rc : A.Rec[(size_t)item * P.rec_words + q];
@@ -569,8 +695,9 @@ __device__ __forceinline__ void slab_apply(const KrylovParams& P, const SlabArgs
         const long long r1 = a + 1 < A.m0 ? acc[1].fold() : 0;
         if (act) {
             A.Wp[item] = make_longlong2(r0, r1);
-            dots.add(c.x, c0, split31(r0));
-            dots.add(c.z, c1, split31(r1));
+            dots.add(c0, split31(r0));
+            dots.add(c1, split31(r1));
+            dots.flush();
         }
     }
 }
@@ -699,7 +826,7 @@ struct VecHist {
     double2 c, m;
 };
 
-// Coefficients of a pole's update as fixed point: {hi, (float)hi, (float)lo}
+// Coefficients of a pole's update as fixed point: {hi, (float)hi, (float)lo, lo}
 // of Re w, Im w, Re v, Im v for every vector, scaled to an l1 norm below 1/2
 // so that no sum overflows.
 __device__ void vec_coefs(const VecHist* hist, int n, int s0, PoleState& s, int pole, int4* co, VecHead* head) {
@@ -729,7 +856,7 @@ __device__ void vec_coefs(const VecHist* hist, int n, int s0, PoleState& s, int 
                 const double f[4] = {w.x / sw, w.y / sw, v.x / sv, v.y / sv};
                 for (int k = 0; k < 4; ++k) {
                     const int2 l = to_limbs(f[k]);
-                    co[4 * j + k] = make_int4(l.x, __float_as_int((float)l.x), __float_as_int((float)l.y), 0);
+                    co[4 * j + k] = make_int4(l.x, __float_as_int((float)l.x), __float_as_int((float)l.y), l.y);
                 }
             }
         }
@@ -749,15 +876,18 @@ __device__ void vec_coefs(const VecHist* hist, int n, int s0, PoleState& s, int 
 }
 
 // x and p of one pole over the slab: fixed-point sums over the kept vectors
-// (the mixed terms in float, 2^-55 of the sum), joined in FP64.  A pair's
-// first point lies at X[xoff(item)], the second beside it.
-template <bool kLast, class F>
+// (the mixed terms in float or in integers), joined in FP64.  A pair's
+// first point lies at Xv[xoff(item)], the second beside it.
+template <bool kLast, bool X, class F>
 __device__ __forceinline__ void vec_update(const SlabArgs& A, int n, const int4* co, const VecHead& h, const int4* Ub,
-                                           double2* X, double2* Pv, F&& xoff) {
+                                           double2* Xv, double2* Pv, F&& xoff) {
     const double sx = h.sw * 0x1p-62, sp = h.sv * 0x1p-62;
     for (int item = threadIdx.x; item < A.n_items; item += blockDim.x) {
         long long hh[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        // (integers: the u_j of one point are entries of nearly orthogonal vectors of
+        // norm 1/4, so the 32 |u_j| sum to less than sqrt(32) / 4, the |lo| terms to 2^62)
         float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        long long mx[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         const int4* up = Ub + item;
 #pragma unroll 2
         for (int j = 0; j < n; ++j) {
@@ -767,14 +897,21 @@ __device__ __forceinline__ void vec_update(const SlabArgs& A, int n, const int4*
 #pragma unroll
             for (int k = 0; k < (kLast ? 2 : 4); ++k) {
                 const int4 c = co[4 * j + k];
-                const float ch = __int_as_float(c.y), cl = __int_as_float(c.z);
                 madw(hh[2 * k], u.x, c.x);
                 madw(hh[2 * k + 1], u.z, c.x);
-                f[2 * k] = fmaf(a0, cl, fmaf(b0, ch, f[2 * k]));
-                f[2 * k + 1] = fmaf(a1, cl, fmaf(b1, ch, f[2 * k + 1]));
+                if constexpr (X) {
+                    madw(mx[2 * k], u.x, c.w);
+                    madw(mx[2 * k], u.y, c.x);
+                    madw(mx[2 * k + 1], u.z, c.w);
+                    madw(mx[2 * k + 1], u.w, c.x);
+                } else {
+                    const float ch = as_float(c.y), cl = as_float(c.z);
+                    f[2 * k] = fmaf(a0, cl, fmaf(b0, ch, f[2 * k]));
+                    f[2 * k + 1] = fmaf(a1, cl, fmaf(b1, ch, f[2 * k + 1]));
+                }
             }
         }
-        double2* x = X + xoff(item);
+        double2* x = Xv + xoff(item);
         double2* p = Pv + 2 * (size_t)item;
         const int pc = item % A.npc;
         const int two = 2 * (pc % A.npx) + 1 < A.m0 ? 2 : 1;
@@ -782,7 +919,9 @@ __device__ __forceinline__ void vec_update(const SlabArgs& A, int n, const int4*
             double v[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                v[k] = (double)((i ? hh[2 * k + 1] : hh[2 * k]) + (long long)((i ? f[2 * k + 1] : f[2 * k]) * 0x1p-31f));
+                v[k] = (double)((i ? hh[2 * k + 1] : hh[2 * k]) +
+                                (X ? (i ? mx[2 * k + 1] : mx[2 * k]) >> 31
+                                   : (long long)((i ? f[2 * k + 1] : f[2 * k]) * 0x1p-31f)));
             double2 xv = make_double2(v[0] * sx, v[1] * sx), pv = make_double2(v[2] * sp, v[3] * sp);
             if (!h.first) {
                 const double2 po = p[i], xo = x[i];
@@ -797,7 +936,7 @@ __device__ __forceinline__ void vec_update(const SlabArgs& A, int n, const int4*
     }
 }
 
-template <int Q, bool kNl>
+template <int Q, bool kNl, bool X>
 __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant__ KrylovParams P) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ KShared S;
@@ -882,7 +1021,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         const KChunk* chk = chunks;
         int n_loc4 = 0, n_rows = 0, n_x = 0;
         if constexpr (kNl) {
-            build_rows(P, m, lo, z0, depth, Q, pitch, pp, SN[0], rows, chunks,
+            build_rows<X>(P, m, lo, z0, depth, Q, pitch, pp, SN[0], rows, chunks,
                        reinterpret_cast<int4*>(slot + P.off_xtab), reinterpret_cast<int*>(Wp),
                        reinterpret_cast<uint2*>(Rec));
             n_loc4 = 4 * SN[0].n_local;
@@ -1003,7 +1142,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         while (!stop) {
             if constexpr (kNl) {
                 // projections of the slab, their sum over the cluster, row factors
-                project(P, U, rows, chk, SN[0].n_chunks, nwp + 1, xtab, stage, acc);
+                project<X>(P, U, rows, chk, SN[0].n_chunks, nwp + 1, xtab, stage, acc);
                 __syncthreads();
                 for (int t = tid; t < n_loc4; t += blockDim.x) {
                     cpart[t] = acc[t];
@@ -1014,15 +1153,15 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                     long long s = 0;
                     for (int r = 0; r < C; ++r)
                         s += __ldcg(reinterpret_cast<const long long*>(slot0 + (size_t)r * P.cta_bytes + P.off_cpart) + t);
-                    cl[t] = tab_limbs(to_limbs((double)s * cf[t]));
+                    cl[t] = tab_limbs<X>(to_limbs((double)s * cf[t]));
                 }
                 __syncthreads();
 #pragma unroll 4
-                for (int t = tid; t < n_rows; t += blockDim.x) ktab[t + 1] = row_factors(rows + t, cl);
+                for (int t = tid; t < n_rows; t += blockDim.x) ktab[t + 1] = row_factors<X>(rows + t, cl);
                 if (tid == 0) ktab[0] = make_int4(0, 0, 0, 0);
                 __syncthreads();
             }
-            Dots dots;
+            Dots<X> dots;
             if (scalar_warp) {
                 // pole recurrences of the step before, while the others compute
                 if (rank == 0 && P.K == 0) {
@@ -1038,8 +1177,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 const int2 g = make_int2(-S.cg.x, -S.cg.y);
                 const int4* up = Up + (size_t)((it - 1 + ring) % ring) * n_items;
                 // (the compiler sees that these tables are in shared memory)
-                if (!kNl || tab_smem) slab_apply<Q, kNl>(P, SA, kt_s, xt_s, up, nwp, g, dots);
-                else slab_apply<Q, kNl>(P, SA, ktab, xtab, up, nwp, g, dots);
+                if (!kNl || tab_smem) slab_apply<Q, kNl, X>(P, SA, kt_s, xt_s, up, nwp, g, dots);
+                else slab_apply<Q, kNl, X>(P, SA, ktab, xtab, up, nwp, g, dots);
             }
             // ---- u.w and w.w over the cluster ------------------------------
             if (!scalar_warp) {
@@ -1147,22 +1286,22 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 __syncthreads();
                 if (S.stop == kMeasure) {
                     const int2 al = S.ca;
-                    const f32x2 alf = lo_hi(al.x, al.y);
+                    const Rhs<X> ar(opaque(al.x), opaque(al.y));
                     const int e = S.e;
-                    Dots sq;
+                    Dots<X> sq;
 #pragma unroll 1
                     for (int item = tid; item < n_items; item += 32 * nwp) {
                         const int d = (int)fdiv((uint32_t)item, SA.div_pc), pc = item - d * npc;
                         const int pb = (int)fdiv((uint32_t)pc, div_px);
                         const int4 u = *reinterpret_cast<const int4*>(U + (d + Q) * pp + pb * pitch + 2 * (pc - pb * npx));
                         const longlong2 w = Wp[item];
-                        const int ax = opaque(al.x);
-                        Acc a0, a1;
-                        a0.mac(u.x, hi_lo(u.x, u.y), ax, alf);
-                        a1.mac(u.z, hi_lo(u.z, u.w), ax, alf);
+                        Acc<X> a0, a1;
+                        a0.mac(Lhs<X>(u.x, u.y), ar);
+                        a1.mac(Lhs<X>(u.z, u.w), ar);
                         const long long t0 = w.x - a0.fold(), t1 = w.y - a1.fold();
-                        sq.add(0, 0, split31(e >= 0 ? t0 << e : t0 >> -e));
-                        sq.add(0, 0, split31(e >= 0 ? t1 << e : t1 >> -e));
+                        sq.add(Lhs<X>(0, 0), split31(e >= 0 ? t0 << e : t0 >> -e));
+                        sq.add(Lhs<X>(0, 0), split31(e >= 0 ? t1 << e : t1 >> -e));
+                        sq.flush();
                     }
                     const long long s = warp_sum4(sq.hh2, sq.l2(), 0LL, 0LL, lane);
                     if (lane < 2) S.part[warp][lane] = s;
@@ -1203,8 +1342,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                     double2* x = P.ckpt ? P.ckpt + P.ckpt_off[(long long)node * P.P + pole]
                                         : Xs + (size_t)pole * 2 * n_items;
                     double2* pv = Ps + (size_t)pole * 2 * n_items;
-                    if (SV.head.last) vec_update<true>(SA, n, SV.co, SV.head, Up, x, pv, vec_index);
-                    else vec_update<false>(SA, n, SV.co, SV.head, Up, x, pv, vec_index);
+                    if (SV.head.last) vec_update<true, X>(SA, n, SV.co, SV.head, Up, x, pv, vec_index);
+                    else vec_update<false, X>(SA, n, SV.co, SV.head, Up, x, pv, vec_index);
                 }
                 s0 = it;
                 k_sync();   // from here the coefficients may be written again
@@ -1212,7 +1351,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
             if (stop) break;
             if (!scalar_warp) {
                 const int2 al = S.ca;
-                const f32x2 alf = lo_hi(al.x, al.y);
+                const Rhs<X> ar(opaque(al.x), opaque(al.y));
                 const int e = S.e;
                 const uint32_t ubase = smem_addr(U);
                 // three pairs at a time: their loads are in flight together
@@ -1231,10 +1370,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                         const int idx = pb * pitch + 2 * (pc - pb * npx);
                         int4* up = reinterpret_cast<int4*>(U + (d + Q) * pp + idx);
                         const int4 u = *up;
-                        const int ax = opaque(al.x);
-                        Acc a0, a1;
-                        a0.mac(u.x, hi_lo(u.x, u.y), ax, alf);
-                        a1.mac(u.z, hi_lo(u.z, u.w), ax, alf);
+                        Acc<X> a0, a1;
+                        a0.mac(Lhs<X>(u.x, u.y), ar);
+                        a1.mac(Lhs<X>(u.z, u.w), ar);
                         const long long t0 = w[j].x - a0.fold(), t1 = w[j].y - a1.fold();
                         const int2 a = split31(e >= 0 ? t0 << e : t0 >> -e), b = split31(e >= 0 ? t1 << e : t1 >> -e);
                         const int4 nu = make_int4(a.x, a.y, b.x, b.y);
@@ -1255,7 +1393,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         }
         // ---- mixed precision: the last step once more, in FP64 ---------------
         double defect = 0.0;
-        if (P.check && !bad) {
+        if (!X && P.check && !bad) {
             double* c = reinterpret_cast<double*>(acc);   // free once the steps are done
             double* part = reinterpret_cast<double*>(cpart);
             double s2 = check_step<Q, kNl>(P, SA, lo, z0, SN[0], c, Up + (size_t)((it - 2 + ring) % ring) * n_items, S.cg, [&]() {
@@ -1375,8 +1513,7 @@ __global__ void k_proj_fixed(long long n_atoms, const int* __restrict__ len, con
             const bool in = u < len[3 * a + warp];
             const double g = in ? gtab[base + u] : 0.0, dg = in ? dtab[base + u] * g : 0.0;
             const int2 x = to_limbs(g * ig), y = to_limbs(dg * id);
-            const int2 a_ = tab_limbs(x), b_ = tab_limbs(y);
-            fx[base + u] = make_int4(a_.x, a_.y, b_.x, b_.y);
+            fx[base + u] = make_int4(x.x, x.y, y.x, y.y);
         }
     }
     __syncthreads();
@@ -1389,7 +1526,7 @@ __global__ void k_proj_fixed(long long n_atoms, const int* __restrict__ len, con
     }
 }
 
-template <int Q, bool kNl>
+template <int Q, bool kNl, bool X>
 int max_clusters(int csz, int block, size_t smem) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = csz;
@@ -1403,17 +1540,17 @@ int max_clusters(int csz, int block, size_t smem) {
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaFuncSetAttribute(k_krylov<Q, kNl>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, k_krylov<Q, kNl>, &cfg) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_krylov<Q, kNl, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, k_krylov<Q, kNl, X>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return n;
 }
 
-template <int Q, bool kNl>
+template <int Q, bool kNl, bool X>
 cudaError_t launch(const KrylovParams& P, int csz, int grid, int block, size_t smem, cudaStream_t stream) {
-    cudaError_t e = cudaFuncSetAttribute(k_krylov<Q, kNl>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_krylov<Q, kNl, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -1427,7 +1564,7 @@ cudaError_t launch(const KrylovParams& P, int csz, int grid, int block, size_t s
     at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_krylov<Q, kNl>, P);
+    return cudaLaunchKernelEx(&cfg, k_krylov<Q, kNl, X>, P);
 }
 
 }  // namespace
@@ -1441,31 +1578,40 @@ size_t kry_vec_bytes(int P) {
 }
 int kry_max_threads() { return kMaxThreads - 32; }
 
+// (clusters of the mixed kernel and of the FP64 one are the same size)
 int kry_max_clusters(int q, int nonlocal, int csz, int block, size_t smem) {
     switch (q * 2 + (nonlocal ? 1 : 0)) {
-        case 2: return max_clusters<1, false>(csz, block, smem);
-        case 3: return max_clusters<1, true>(csz, block, smem);
-        case 4: return max_clusters<2, false>(csz, block, smem);
-        case 5: return max_clusters<2, true>(csz, block, smem);
-        case 6: return max_clusters<3, false>(csz, block, smem);
-        case 7: return max_clusters<3, true>(csz, block, smem);
-        case 8: return max_clusters<4, false>(csz, block, smem);
-        case 9: return max_clusters<4, true>(csz, block, smem);
+        case 2: return max_clusters<1, false, true>(csz, block, smem);
+        case 3: return max_clusters<1, true, true>(csz, block, smem);
+        case 4: return max_clusters<2, false, true>(csz, block, smem);
+        case 5: return max_clusters<2, true, true>(csz, block, smem);
+        case 6: return max_clusters<3, false, true>(csz, block, smem);
+        case 7: return max_clusters<3, true, true>(csz, block, smem);
+        case 8: return max_clusters<4, false, true>(csz, block, smem);
+        case 9: return max_clusters<4, true, true>(csz, block, smem);
     }
     return 0;
 }
 
 cudaError_t launch_krylov(const KrylovParams& P, int q, int nonlocal, int csz, int grid, int block, size_t smem,
                           cudaStream_t stream) {
-    switch (q * 2 + (nonlocal ? 1 : 0)) {
-        case 2: return launch<1, false>(P, csz, grid, block, smem, stream);
-        case 3: return launch<1, true>(P, csz, grid, block, smem, stream);
-        case 4: return launch<2, false>(P, csz, grid, block, smem, stream);
-        case 5: return launch<2, true>(P, csz, grid, block, smem, stream);
-        case 6: return launch<3, false>(P, csz, grid, block, smem, stream);
-        case 7: return launch<3, true>(P, csz, grid, block, smem, stream);
-        case 8: return launch<4, false>(P, csz, grid, block, smem, stream);
-        case 9: return launch<4, true>(P, csz, grid, block, smem, stream);
+    switch ((q * 2 + (nonlocal ? 1 : 0)) * 2 + (P.check ? 0 : 1)) {
+        case 4: return launch<1, false, false>(P, csz, grid, block, smem, stream);
+        case 5: return launch<1, false, true>(P, csz, grid, block, smem, stream);
+        case 6: return launch<1, true, false>(P, csz, grid, block, smem, stream);
+        case 7: return launch<1, true, true>(P, csz, grid, block, smem, stream);
+        case 8: return launch<2, false, false>(P, csz, grid, block, smem, stream);
+        case 9: return launch<2, false, true>(P, csz, grid, block, smem, stream);
+        case 10: return launch<2, true, false>(P, csz, grid, block, smem, stream);
+        case 11: return launch<2, true, true>(P, csz, grid, block, smem, stream);
+        case 12: return launch<3, false, false>(P, csz, grid, block, smem, stream);
+        case 13: return launch<3, false, true>(P, csz, grid, block, smem, stream);
+        case 14: return launch<3, true, false>(P, csz, grid, block, smem, stream);
+        case 15: return launch<3, true, true>(P, csz, grid, block, smem, stream);
+        case 16: return launch<4, false, false>(P, csz, grid, block, smem, stream);
+        case 17: return launch<4, false, true>(P, csz, grid, block, smem, stream);
+        case 18: return launch<4, true, false>(P, csz, grid, block, smem, stream);
+        case 19: return launch<4, true, true>(P, csz, grid, block, smem, stream);
     }
     return cudaErrorInvalidValue;
 }

@@ -20,22 +20,23 @@ constexpr int kKryMaxDepth = 40;   // planes of a CTA's slab (bounds the exact p
 
 struct KrylovParams {
     // operator A = (H_R - shift) / scale, weights in two signed 31-bit limbs
-    // (value = hi 2^-31 + lo 2^-62), wf the pair {(float)lo, (float)hi}
+    // (value = hi 2^-31 + lo 2^-62), wf the pair {(float)lo, (float)hi}; the
+    // mixed-precision kernel takes wf, the FP64 one wl
     int n[3];
     int periodic[3];
     const double* V;
     double scale, shift;
-    int wh[3][kKryMaxQ];
+    int wh[3][kKryMaxQ], wl[3][kKryMaxQ];
     unsigned long long wf[3][kKryMaxQ];
     // nonlocal projectors
     long long n_atoms;
     const int* proj_i0;
     const int* proj_len;
     const unsigned char* proj_rows;
-    const int4* proj_fx;           // [atom][axis][kMaxProjWin] unit tables: g (hi, (float)lo), d g (hi, (float)lo), halved
+    const int4* proj_fx;           // [atom][axis][kMaxProjWin] unit tables: g (hi, lo), d g (hi, lo), halved
     const double* proj_fxc;        // [atom][4] 64 E_l C_l^2 of the unit tables
     int rec_words;                 // 4 projector rows per word and region point
-    // FP64 operator of the final check of a mixed solve
+    // mixed precision: FP32 mixed terms, and the FP64 operator of the final check
     int check;
     double coef[3][kKryMaxQ];
     double dV, e_s, e_p;

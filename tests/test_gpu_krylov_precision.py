@@ -1,0 +1,41 @@
+"""FP64 calls on the node-shared kernel are as exact as on the FP64 kernels."""
+import numpy as np
+import pytest
+
+from synthetic import make_workload
+
+pytestmark = pytest.mark.gpu
+
+
+def _spiked(spike, nodes=24, s=8):
+    """Bulk cell whose potential is `spike` at one point outside every region:
+    the regions' operators are untouched, the fixed-point scale follows it."""
+    from paper_1907_02604_gb300 import Hamiltonian
+    w = make_workload("bulk_mixed").subset(np.arange(nodes))
+    w.halfwidth[:] = s
+    n = np.array(w.shape)
+    c = w.node_coords()
+    for g in range(0, w.n_grid, 977):
+        p = np.array([g % n[0], g // n[0] % n[1], g // (n[0] * n[1])])
+        d = np.abs(c - p)
+        if (np.minimum(d, n - d).max(1) > s + 4).all():
+            break
+    ham = Hamiltonian.from_workload(w)
+    if spike:
+        V = ham.potential()
+        V[g] = spike
+        ham.set_potential(V)
+    return w, ham
+
+
+@pytest.mark.parametrize("spike", [0.0, 400.0])
+def test_rules_as_exact_as_the_fp64_kernel(spike):
+    """The two kernels' lowest nodes.  Both round the Jacobi matrix (entries of
+    10 to 20 Ha) and its QR to half an ulp, 2e-15 Ha; nodes of small weight
+    answer with about three times that, 5e-15 a side.  Products cut to 2^-57 of
+    the scale were off by 1e-13 Ha in alpha after 40 steps."""
+    from paper_1907_02604_gb300 import lssgq_rules
+    w, ham = _spiked(spike)
+    lam = [lssgq_rules(ham, w.nodes, w.halfwidth, K=40, precision="fp64", block=b).lam.cpu().numpy()[:, :6]
+           for b in (0, 1024)]
+    assert np.sqrt(np.mean((lam[0] - lam[1]) ** 2)) <= 1.2e-14

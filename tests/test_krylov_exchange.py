@@ -12,6 +12,7 @@ import numpy as np
 import pytest
 
 from synthetic import make_workload
+from tests.gpu_helpers import rel_err
 
 SRC = os.path.join(os.path.dirname(__file__), "..", "paper_1907_02604_gb300", "csrc", "md_krylov.cu")
 
@@ -29,8 +30,9 @@ def test_check_has_a_mailbox_word_of_its_own():
 
 @pytest.mark.gpu
 def test_mixed_check_on_thin_slabs():
-    """Without projectors a mixed call runs the FP64 call's kernel and adds the
-    check: the values are the same bits, run after run."""
+    """Without projectors every sum of a mixed call has a fixed order: the same
+    bits run after run, and those of the FP64 call to 1e-11 (x_jp(j) is in error
+    by tol^2 / Im z and by rounding)."""
     from paper_1907_02604_gb300 import Hamiltonian, SolverOptions, density, make_poles
     hw = [0, 1, 2, 3, 4, 5, 6, 7, 8, 0, 1, 1, 3, 6]   # one point among 17^3: CTAs without a plane
     w = make_workload("tiny", shape=(24, 24, 24), n_nodes=len(hw), n_atoms=6, spacing=(0.6, 0.6, 0.6), fd_order=4,
@@ -39,7 +41,10 @@ def test_mixed_check_on_thin_slabs():
     ham = Hamiltonian.from_workload(w)
     z, wt = make_poles(w.kT, w.mu, *ham.spectral_bounds(), w.n_poles)
     want = density(ham, z, wt, w.nodes, w.halfwidth, SolverOptions(tol=1e-10), energy=True)
+    first = None
     for _ in range(30):
         rho, e, st = density(ham, z, wt, w.nodes, w.halfwidth, SolverOptions(tol=1e-10, precision="mixed"), energy=True)
         assert st["n_converged"] == w.n_systems
-        assert rho.equal(want[0]) and e.equal(want[1])
+        first = first or (rho, e)
+        assert rho.equal(first[0]) and e.equal(first[1])
+    assert rel_err(first[0].cpu().numpy(), want[0].cpu().numpy()) <= 1e-11
