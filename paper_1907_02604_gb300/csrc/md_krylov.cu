@@ -1458,8 +1458,16 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
         if (rank == 0 && scalar_warp) {
             if (P.K == 0 && it > proc) poles(it);
             if (P.K > 0) {
+                // a potential that is not finite: so is the Jacobi matrix, and its QR fails
+                if (bad == 3) {
+                    const double nan = __longlong_as_double(0x7ff8000000000000LL);
+                    for (int k = lane; k < P.K; k += 32) {
+                        P.alpha[(long long)node * P.K + k] = nan;
+                        P.beta[(long long)node * P.K + k] = nan;
+                    }
+                }
                 if (lane == 0) {
-                    P.k_used[node] = bad ? 0 : it;
+                    P.k_used[node] = bad == 3 ? P.K : (bad ? 0 : it);
                     P.node_status[node] = bad == 1 ? 1 : (stop == 2 ? 4 : 0);
                 }
             } else {
