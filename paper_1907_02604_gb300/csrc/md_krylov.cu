@@ -459,7 +459,7 @@ __device__ void build_rows(const KrylovParams& P, const int m[3], const int lo[3
                         const int pos = atomicAdd(cnt + item0 + pr, 1);
                         if (pos < 2 * P.rec_words)
                             rec[(size_t)(item0 + pr) * 2 * P.rec_words + pos] =
-                                make_uint2((uint32_t)(id + 1) | (f0 ? x << 16 : 0u), f1 ? x + 1 : 0u);
+                                make_uint2((uint32_t)(id + 1) | (f0 ? x << 16 : 0u), (f1 ? x + 1 : 0u) | (uint32_t)k << 16);
                         else S.over = 1;
                     }
                 }
@@ -487,6 +487,22 @@ __device__ void build_rows(const KrylovParams& P, const int m[3], const int lo[3
                 for (int u = lane; u < P.win_x; u += 32) xtab[1 + tab * P.win_x + u] = tab_entry<X>(tx[u]);
             }
         }
+    }
+    __syncthreads();
+    // A pair's entries by atom and row, whichever warp was first: the mixed
+    // terms of mixed precision are floats, whose sum depends on the order.
+    // (Row ids ascend within an atom; the atom's slot rides in the second word.)
+    for (int t = threadIdx.x; t < depth * m[1] * npx; t += blockDim.x) {
+        uint2* r = rec + (size_t)t * 2 * P.rec_words;
+        const int n = min(cnt[t], 2 * P.rec_words);
+        auto key = [](uint2 e) { return (e.y & 0xffff0000u) | (e.x & 0xffffu); };
+        for (int i = 1; i < n; ++i) {
+            const uint2 e = r[i];
+            int j = i;
+            for (; j > 0 && key(r[j - 1]) > key(e); --j) r[j] = r[j - 1];
+            r[j] = e;
+        }
+        for (int i = 0; i < n; ++i) r[i].y &= 0xffffu;
     }
     __syncthreads();
 }
@@ -706,8 +722,10 @@ __device__ __forceinline__ double limbs(int hi, int lo) { return fma((double)hi,
 
 // Sum over the slab of (A u - g u_prev - w)^2, everything evaluated in FP64
 // from the FP64 potential and projector values: how far the fixed-point step
-// just taken is from the operator's.  c: [n_local][4] doubles, zeroed here;
-// xsum exchanges them over the cluster.
+// just taken is from the operator's.  c: [n_local][4] projections, zeroed here;
+// xsum exchanges them over the cluster.  A CTA's share is summed in units of
+// 2^-60 / sqrt(dV) (a projector has norm 1 / sqrt(dV) and ||u|| < 1/4), so that
+// it does not depend on the order of the atomics.
 template <int Q, bool kNl, class F>
 __device__ __noinline__ double check_step(const KrylovParams& P, const SlabArgs& A, const int lo[3], int z0,
                                           const KSharedNl& S, double* c, const int4* u_prev, int2 g2,
@@ -731,7 +749,9 @@ __device__ __noinline__ double check_step(const KrylovParams& P, const SlabArgs&
         return -1;
     };
     if constexpr (kNl) {
-        for (int t = threadIdx.x; t < 4 * S.n_local; t += blockDim.x) c[t] = 0.0;
+        unsigned long long* ci = reinterpret_cast<unsigned long long*>(c);
+        const double unit = sqrt(P.dV) * 0x1p60;
+        for (int t = threadIdx.x; t < 4 * S.n_local; t += blockDim.x) ci[t] = 0;
         __syncthreads();
         for (int item = threadIdx.x; item < A.n_items; item += blockDim.x) {
             int d, b, a;
@@ -744,13 +764,14 @@ __device__ __noinline__ double check_step(const KrylovParams& P, const SlabArgs&
                     const int s = slot_of(P.pl_atom[e]);
                     if (s < 0) continue;
                     const double2 p = P.pl_val64[2 * e], q = P.pl_val64[2 * e + 1];
-                    atomicAdd(c + 4 * s, p.x * u);
-                    atomicAdd(c + 4 * s + 1, p.y * u);
-                    atomicAdd(c + 4 * s + 2, q.x * u);
-                    atomicAdd(c + 4 * s + 3, q.y * u);
+                    const double f[4] = {p.x, p.y, q.x, q.y};
+                    for (int l = 0; l < 4; ++l)
+                        atomicAdd(ci + 4 * s + l, (unsigned long long)__double2ll_rn(f[l] * u * unit));
                 }
             }
         }
+        __syncthreads();
+        for (int t = threadIdx.x; t < 4 * S.n_local; t += blockDim.x) c[t] = (double)(long long)ci[t] / unit;
         xsum();
     }
     const double inv = 1.0 / P.scale;
