@@ -245,6 +245,8 @@ namespace {
 // ---------------------------------------------------------------------------
 
 constexpr int kKryClasses = 12;   // region-size classes of one batch, launched side by side
+constexpr size_t kKryCounters = kKryClasses * sizeof(unsigned int) + sizeof(unsigned long long);   // and the start time
+static_assert(kKryClasses % 2 == 0, "start time aligned");
 constexpr int kKryStreams = 12;   // the caller's stream and those of KrySide: a class to each
 
 }  // namespace
@@ -527,6 +529,7 @@ void kry_scratch(std::vector<KryClass>& cls, char* base, const int* list, unsign
         P.list = list + first[k];
         P.nodes = nodes;
         P.work_counter = counters + k;
+        P.t_start = (unsigned long long*)(counters + kKryClasses);
     }
 }
 
@@ -917,9 +920,9 @@ struct FusedArgs {
     const long long* dm_off;
 };
 
-// Reset the work counters, solve, accumulate rho and e.
+// Reset the work counters and the start time, solve, accumulate rho and e.
 cudaError_t plan_enqueue(md_plan* pl, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(pl->d_counter, 0, kKryClasses * sizeof(unsigned int), s);
+    cudaError_t e = cudaMemsetAsync(pl->d_counter, 0, kKryCounters, s);
     if (e != cudaSuccess) return e;
     if (!pl->kry.empty()) e = kry_launch(pl->kry, *pl->H, pl->side, s);
     else e = launch_shape(pl, pl->P, Shape{pl->variant, pl->block, pl->per_sm, pl->cluster}, pl->grid, s);
@@ -1087,7 +1090,7 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     PTRY(dmalloc(&pl->d_xsrc, n_sys * sizeof(double2)));
     PTRY(dmalloc(&pl->d_z, Pn * sizeof(double2)));
     PTRY(dmalloc(&pl->d_w, Pn * sizeof(double2)));
-    PTRY(dmalloc(&pl->d_counter, kKryClasses * sizeof(unsigned int)));
+    PTRY(dmalloc(&pl->d_counter, kKryCounters));
     if (kry) {   // the work list of the classes takes the place of the system list
         static_assert(sizeof(SysDesc) >= sizeof(int), "node list fits the system list");
         std::memcpy(sys.data(), korder.data(), nn * sizeof(int));
@@ -1985,7 +1988,7 @@ extern "C" md_status md_lssgq_rules(const md_hamiltonian* ham, const md_nodes* n
     if (kry) std::memcpy(sys.data(), korder.data(), nn * sizeof(int));
     LTRY(cudaMemcpyAsync(d_sys, sys.data(), nn * sizeof(SysDesc), cudaMemcpyHostToDevice, s));
     LTRY(cudaMemcpyAsync(d_nodes, R.desc.data(), nn * sizeof(NodeDesc), cudaMemcpyHostToDevice, s));
-    LTRY(cudaMemsetAsync(d_counter, 0, kKryClasses * sizeof(unsigned int), s));
+    LTRY(cudaMemsetAsync(d_counter, 0, kKryCounters, s));
     LTRY(cudaMemsetAsync(d_kused, 0, nn * sizeof(int), s));
     P.sys = d_sys;
     P.nodes = d_nodes;

@@ -963,11 +963,21 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
     __shared__ KShared S;
     __shared__ KSharedVec SV;
     __shared__ KSharedNl SN[1];   // untouched (and dropped) without projectors
-    const uint64_t t_start = global_time_ns();
     const int C = (int)k_nrank(), rank = (int)k_rank();
     const int nwp = (int)(blockDim.x >> 5) - 1;  // warps that compute points
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool scalar_warp = warp == nwp;
+    // the budget runs from the first CTA of any of the call's launches
+    uint64_t t_start = 0;
+    if (P.timeout_ns && rank == 0 && scalar_warp && lane == 0) {
+        const uint64_t now = global_time_ns(), first = atomicCAS(P.t_start, 0ULL, (unsigned long long)now);
+        t_start = first ? first : now;
+    }
+    auto timed_out = [&]() {   // lane 0 of rank 0's scalar warp
+        if (!P.timeout_ns) return false;
+        const uint64_t now = global_time_ns();
+        return now > t_start && now - t_start > P.timeout_ns;
+    };
     int2* U = reinterpret_cast<int2*>(dsm);
     char* slot = P.scratch + (size_t)blockIdx.x * P.cta_bytes;
     char* slot0 = P.scratch + (size_t)(blockIdx.x - rank) * P.cta_bytes;   // rank 0's slot
@@ -1188,11 +1198,11 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 if (rank == 0 && P.K == 0) {
                     if (it > proc) poles(it);
                     int flag = all_done ? 1 : 0;
-                    if (P.timeout_ns && global_time_ns() - t_start > P.timeout_ns) flag = 2;
+                    if (lane == 0 && timed_out()) flag = 2;
                     flag = __shfl_sync(0xffffffffu, flag, 0);
                     if (lane == 0) S.stop = flag;
                 } else if (rank == 0) {
-                    if (lane == 0 && P.timeout_ns && global_time_ns() - t_start > P.timeout_ns) S.stop = 2;
+                    if (lane == 0 && timed_out()) S.stop = 2;
                 }
             } else {
                 const int2 g = make_int2(-S.cg.x, -S.cg.y);

@@ -49,6 +49,7 @@ struct KrylovParams {
     const NodeDesc* nodes;
     unsigned int* work_counter;
     unsigned long long timeout_ns;
+    unsigned long long* t_start;   // when the call's first CTA ran (0: not yet), shared by its launches
     // per-CTA scratch layout
     char* scratch;
     size_t cta_bytes;

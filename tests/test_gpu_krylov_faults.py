@@ -31,3 +31,28 @@ def test_rules_of_a_potential_that_is_not_finite(precision, block):
     # one node a rule: nothing to iterate, and the NaN is the answer
     lam = lssgq_rules(ham, w.nodes, w.halfwidth, K=1, precision=precision, block=block).lam.cpu().numpy()
     assert np.isnan(lam[0, 0]) and lam[1, 0] == good[1, 0]
+
+
+def test_time_budget_of_many_region_sizes():
+    """Twelve classes of region size, each with nodes for the whole device, and
+    poles in the middle of the spectrum that none of them can reach: the budget
+    is the call's, not each class's.  On top of it every node left takes its
+    set-up and one step, well under 0.1 ms on a tenth of the device: 0.2 s for
+    all."""
+    import time
+    import torch
+    from paper_1907_02604_gb300 import SolverOptions, density
+    from paper_1907_02604_gb300._lib import MacroDFTError
+    sizes = np.repeat(np.arange(3, 15), 160)
+    w, ham = _system(shape=(36, 36, 36), n_nodes=len(sizes), n_atoms=4, spacing=(0.5, 0.5, 0.5), fd_order=8)
+    w.halfwidth = sizes.astype(np.int32)
+    z = np.array([10.0, 12.0, 14.0, 16.0]) + 1e-9j
+
+    def run(budget):
+        with pytest.raises(MacroDFTError, match="MD_ERR_TIMEOUT"):
+            density(ham, z, np.ones(4), w.nodes, w.halfwidth, SolverOptions(tol=1e-12, maxit=10 ** 8, timeout_s=budget))
+        torch.cuda.synchronize()
+    run(1e-6)   # allocations of a first call
+    t = time.time()
+    run(0.3)
+    assert time.time() - t < 0.5
