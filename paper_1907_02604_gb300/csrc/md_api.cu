@@ -277,6 +277,22 @@ double kry_scale(const Ham& H) {
     return std::exp2(std::ceil(std::log2(need)) + 0.0);
 }
 
+// Whether the fixed-point operator serves a call of this precision.  Steps of
+// 2^-62 of the scale are absolute: a potential that is high anywhere on the
+// grid coarsens every region's operator, where FP64's steps follow each entry.
+// FP64 calls take it up to 64 times the stencil's own scale.  Against the FP64
+// kernels on regions of the bulk cell (scale 64; 17^3 to 21^3, densities of 40-point
+// rules differ by 6e-14 from rounding alone): scale 4,096 7e-14, 32,768 8e-13,
+// 2^18 3e-11, 2^25 1e-7; solved densities 2e-13, 3e-13, 2e-12, 6e-9.  Mixed
+// calls, whose per-pole kernels hold V in FP32, take it at any scale.
+bool kry_in_range(const Ham& H, int precision) {
+    const double scale = kry_scale(H);
+    double rad = 0.0;
+    for (int d = 0; d < 3; ++d)
+        for (int o = 0; o < H.q; ++o) rad += 2.0 * std::fabs(H.coef[d][o]);
+    return scale > 0.0 && (precision == MD_PREC_MIXED || scale <= 64.0 * 2.0 * rad);
+}
+
 void kry_operator(KrylovParams& P, const Ham& H, double scale) {
     P.scale = scale;
     P.shift = H.diag;
@@ -621,6 +637,13 @@ struct md_plan {
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     bool launched = false;
     std::vector<md::KryClass> kry;     // node-shared Krylov solve: one launch per size class
+    // what a replayed node-shared plan was made from (see plan_launch)
+    const md_hamiltonian* ham = nullptr;
+    std::vector<double> z, w;
+    std::vector<int64_t> node;
+    std::vector<int32_t> halfwidth;
+    md_solver_opts opts;
+    md_workspace* ckpt = nullptr;
     md::KrySide side;
 };
 
@@ -1057,7 +1080,7 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     // fixed-point ones on the bulk cell)
     const bool kry = !per_pole && opts.kernel == 0 && opts.block == 0 && opts.ctas_per_sm == 0 && Pn <= kKryMaxPoles &&
                      (Pn > 1 || opts.precision == MD_PREC_FP64) && !(ms && opts.precision == MD_PREC_MIXED) &&
-                     kry_scale(H) > 0.0 && kry_classes(H, R, korder, kfirst, kshape, kdims);
+                     kry_in_range(H, opts.precision) && kry_classes(H, R, korder, kfirst, kshape, kdims);
     const bool kvec = ckpt || fused;   // the solution vectors are needed
     const size_t kneed = kry ? kry_params(H, kfirst, kshape, kdims, pl->kry, kvec ? Pn : 0, !ckpt) : 0;
     if (direct && !kry) PTRY(cudaStreamCreateWithFlags(&pl->cap, cudaStreamNonBlocking));   // for tuning trials
@@ -1304,6 +1327,15 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
         *out = pl;
         return MD_OK;
     }
+    if (kry) {
+        pl->ham = ham;
+        pl->z.assign(poles->z, poles->z + 2 * Pn);
+        pl->w.assign(poles->w, poles->w + 2 * Pn);
+        pl->node.assign(nodes->node, nodes->node + nn);
+        pl->halfwidth.assign(nodes->halfwidth, nodes->halfwidth + nn);
+        pl->opts = *opts_in;
+        pl->ckpt = ckpt;
+    }
     // capture the same once; launches replay it
     PTRY(plan_capture(pl));
 #undef PTRY
@@ -1316,9 +1348,19 @@ md_status plan_launch(md_plan* pl, cudaStream_t stream) {
     if (pl->n_sys == 0) return MD_OK;
     if (!pl->kry.empty()) {
         // md_hamiltonian_set_potential may have moved the spectral bounds
-        // that fix the scale of the fixed-point operator
+        // that fix the scale of the fixed-point operator, or left its range:
+        // then the plan goes on with the per-pole kernels
         const double scale = kry_scale(*pl->H);
-        if (scale > 0.0 && scale != pl->kry[0].P.scale) {
+        if (!kry_in_range(*pl->H, pl->precision)) {
+            const md_poles p{pl->Pn, pl->z.data(), pl->w.data()};
+            const md_nodes n{(int64_t)pl->nn, pl->node.data(), pl->halfwidth.data()};
+            md_plan* next = nullptr;
+            const md_status st = plan_create(pl->ham, &p, &n, &pl->opts, pl->rho_out, pl->e_out, pl->ckpt, false, stream,
+                                             &next, nullptr, false, false, true);
+            if (st != MD_OK) return st;
+            std::swap(*pl, *next);
+            plan_free(next);
+        } else if (scale != pl->kry[0].P.scale) {
             for (KryClass& c : pl->kry) kry_operator(c.P, *pl->H, scale);
             PLAN_TRY(plan_capture(pl));
         }
@@ -1950,7 +1992,8 @@ extern "C" md_status md_lssgq_rules(const md_hamiltonian* ham, const md_nodes* n
     std::vector<NodeDesc> kdims;
     std::vector<KryClass> kcls;
     // (FP32 vectors keep their own kernel: at 24 B a point-step it is faster)
-    const bool kry = opts->precision == MD_PREC_FP64 && opts->block == 0 && kry_scale(H) > 0.0 && kry_classes(H, R, korder, kfirst, kshape, kdims);
+    const bool kry = opts->precision == MD_PREC_FP64 && opts->block == 0 && kry_in_range(H, MD_PREC_FP64) &&
+                     kry_classes(H, R, korder, kfirst, kshape, kdims);
     const size_t need = kry ? kry_params(H, kfirst, kshape, kdims, kcls) : P.slot_bytes * (size_t)grid;
     if (need > H.scratch_bytes) {
         LTRY(cudaStreamSynchronize(s));

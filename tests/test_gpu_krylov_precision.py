@@ -39,3 +39,43 @@ def test_rules_as_exact_as_the_fp64_kernel(spike):
     lam = [lssgq_rules(ham, w.nodes, w.halfwidth, K=40, precision="fp64", block=b).lam.cpu().numpy()[:, :6]
            for b in (0, 1024)]
     assert np.sqrt(np.mean((lam[0] - lam[1]) ** 2)) <= 1.2e-14
+
+
+def _both(f):
+    per_pole = dict(kernel="generic", block=256, ctas_per_sm=1)
+    return [x.cpu().numpy() for x in (f({}), f(per_pole))]
+
+
+@pytest.mark.parametrize("spike", [1e5, 1e7])
+def test_potential_that_is_high_elsewhere(spike):
+    """FP64 calls whose regions do not touch a high potential: rules are the FP64
+    kernel's, densities and a plan made before the potential rose those of the
+    per-pole kernels to 1e-11 (tol 1e-11; x_jp(j) is in error by tol^2 / Im z
+    and by rounding, a few 1e-13).  Steps of 2^-62 of the scale were off by up to
+    1e-7 and 6e-9."""
+    import torch
+    from paper_1907_02604_gb300 import Plan, SolverOptions, density, lssgq_rules, make_poles
+    w, ham = _spiked(0.0, nodes=8)
+    low = ham.potential()
+    _, high = _spiked(spike, nodes=8)
+    z, wt = make_poles(0.01, 0.2, -10.0, 46.0, 16)
+    o = SolverOptions(tol=1e-11)
+    plan = Plan(ham, z, wt, w.nodes, w.halfwidth, o)
+    plan.launch()
+    plan.stats()
+    before = plan.rho.clone()
+    V = high.potential()
+    ham.set_potential(V)
+    lam = [lssgq_rules(ham, w.nodes, w.halfwidth, K=40, precision="fp64", block=b).lam for b in (0, 1024)]
+    assert torch.equal(*lam)
+    r, ref = _both(lambda k: density(ham, z, wt, w.nodes, w.halfwidth, SolverOptions(tol=1e-11, **k))[0])
+    assert np.abs(r - ref).max() <= 1e-11 * np.abs(ref).max()
+    for _ in range(2):
+        plan.launch()
+        st = plan.stats()
+        assert st["n_converged"] == 8 * 16
+        assert np.abs(plan.rho.cpu().numpy() - ref).max() <= 1e-11 * np.abs(ref).max()
+    ham.set_potential(low)
+    plan.launch()
+    plan.stats()
+    assert np.abs((plan.rho - before).cpu().numpy()).max() <= 1e-11 * np.abs(ref).max()
