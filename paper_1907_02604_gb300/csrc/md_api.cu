@@ -1992,15 +1992,25 @@ extern "C" md_status md_lssgq_rules(const md_hamiltonian* ham, const md_nodes* n
     std::vector<NodeDesc> kdims;
     std::vector<KryClass> kcls;
     // (FP32 vectors keep their own kernel: at 24 B a point-step it is faster)
-    const bool kry = opts->precision == MD_PREC_FP64 && opts->block == 0 && kry_in_range(H, MD_PREC_FP64) &&
-                     kry_classes(H, R, korder, kfirst, kshape, kdims);
-    const size_t need = kry ? kry_params(H, kfirst, kshape, kdims, kcls) : P.slot_bytes * (size_t)grid;
+    bool kry = opts->precision == MD_PREC_FP64 && opts->block == 0 && kry_in_range(H, MD_PREC_FP64) &&
+               kry_classes(H, R, korder, kfirst, kshape, kdims);
+    size_t need = kry ? kry_params(H, kfirst, kshape, kdims, kcls) : P.slot_bytes * (size_t)grid;
     if (need > H.scratch_bytes) {
         LTRY(cudaStreamSynchronize(s));
         if (H.scratch) cudaFree(H.scratch);
         H.scratch = nullptr;
         H.scratch_bytes = 0;
-        LTRY(cudaMalloc(&H.scratch, need));
+        cudaError_t e = cudaMalloc(&H.scratch, need);
+        if (e == cudaErrorMemoryAllocation && kry) {
+            // with projectors its records take three times the FP64 kernel's
+            // slots (380 MB against 131 for 33^3 regions): that runs where they
+            // cannot be had
+            cudaGetLastError();
+            kry = false;
+            need = P.slot_bytes * (size_t)grid;
+            e = cudaMalloc(&H.scratch, need);
+        }
+        LTRY(e);
         H.scratch_bytes = need;
     }
     P.scratch = (char*)H.scratch;

@@ -56,3 +56,26 @@ def test_time_budget_of_many_region_sizes():
     t = time.time()
     run(0.3)
     assert time.time() - t < 0.5
+
+
+def test_rules_on_a_device_that_is_nearly_full():
+    """FP64 rules of 33^3 regions with projectors need 131 MB on the FP64 kernel
+    and 380 on the node-shared one: with 240 MB free they come from the former."""
+    import torch
+    from paper_1907_02604_gb300 import Hamiltonian, lssgq_rules
+    w = make_workload("bulk_mixed").subset(np.arange(160))
+    tw, tham = _system(shape=(20, 20, 20), n_nodes=2, s=4, n_atoms=2, spacing=(0.5, 0.5, 0.5), nonlocal_proj=True, fd_order=8)
+    for block in (0, 1024):   # both kernels loaded
+        lssgq_rules(tham, tw.nodes, tw.halfwidth, K=4, block=block)
+    ref = Hamiltonian.from_workload(w)
+    want = lssgq_rules(ref, w.nodes, w.halfwidth, K=8, block=1024).lam
+    ref.close()
+    ham = Hamiltonian.from_workload(w)
+    torch.cuda.synchronize()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - 240 * 10 ** 6, dtype=torch.uint8, device="cuda")
+    try:
+        lam = lssgq_rules(ham, w.nodes, w.halfwidth, K=8).lam
+        assert torch.equal(lam, want)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
