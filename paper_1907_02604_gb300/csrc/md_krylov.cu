@@ -995,6 +995,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
     KChunk* const chunks = reinterpret_cast<KChunk*>(slot + P.off_chunk);
     long long* const cpart = reinterpret_cast<long long*>(slot + P.off_cpart);
 
+    k_sync();   // every CTA of the cluster runs: its shared memory may be written from here on
     for (;;) {
         if (rank == 0 && tid == 0) {
             const int w = (int)atomicAdd(P.work_counter, 1u);

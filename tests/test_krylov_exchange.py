@@ -28,6 +28,14 @@ def test_check_has_a_mailbox_word_of_its_own():
     assert not stored & read
 
 
+def test_cluster_meets_before_the_first_remote_store():
+    """Shared memory of another CTA may be written once that CTA runs."""
+    src = open(SRC).read()
+    kernel = src[src.index("k_krylov(const __grid_constant__ KrylovParams P) {"):]
+    start = kernel[:kernel.index("st.shared::cluster")]
+    assert "k_sync();" in start
+
+
 @pytest.mark.gpu
 def test_mixed_check_on_thin_slabs():
     """Without projectors every sum of a mixed call has a fixed order: the same
