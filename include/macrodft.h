@@ -126,7 +126,10 @@ typedef struct {
                               the previous one restarts the Krylov recurrence.
                               The node-shared kernel recomputes its last step in
                               FP64 once per node and adds the defect it finds to
-                              every residual before it declares convergence */
+                              every residual before it declares convergence; with
+                              a tolerance near that defect it forms its products
+                              as in FP64 calls, without the check, and below its
+                              steps the per-pole kernels run */
     double timeout_s;      /* device wall-clock budget for the call, 0 = none */
     int32_t block;         /* threads per CTA; 0 = library choice */
     int32_t ctas_per_sm;   /* resident CTAs per SM; 0 = library choice.  With
@@ -174,7 +177,8 @@ typedef struct {
     int64_t total_iters;       /* sum over systems */
     int64_t total_point_iters; /* sum over systems of iters * region points */
     int64_t reliable_updates;  /* mixed: FP64 residual recomputations, summed over
-                                  systems (node-shared kernel: one per system) */
+                                  systems (node-shared kernel: one per system, none
+                                  with a tolerance that takes its FP64 form) */
     double max_resid;          /* max final relative residual */
     double kernel_ms;          /* device time of the solver launch */
 } md_stats;

@@ -277,20 +277,35 @@ double kry_scale(const Ham& H) {
     return std::exp2(std::ceil(std::log2(need)) + 0.0);
 }
 
-// Whether the fixed-point operator serves a call of this precision.  Steps of
-// 2^-62 of the scale are absolute: a potential that is high anywhere on the
-// grid coarsens every region's operator, where FP64's steps follow each entry.
-// FP64 calls take it up to 64 times the stencil's own scale.  Against the FP64
-// kernels on regions of the bulk cell (scale 64; 17^3 to 21^3, densities of 40-point
-// rules differ by 6e-14 from rounding alone): scale 4,096 7e-14, 32,768 8e-13,
-// 2^18 3e-11, 2^25 1e-7; solved densities 2e-13, 3e-13, 2e-12, 6e-9.  Mixed
-// calls, whose per-pole kernels hold V in FP32, take it at any scale.
-bool kry_in_range(const Ham& H, int precision) {
+// Which form of the fixed-point kernel serves a call: FP32 mixed terms, integer
+// ones, or neither.  Its steps are absolute, 2^-62 of the scale with integer
+// mixed terms and 2^-57 with FP32 ones, where FP64's follow each entry: a
+// potential that is high anywhere on the grid coarsens every region's operator.
+//   FP64 calls take integers up to 64 times the stencil's own scale.  Against the
+// FP64 kernels on regions of the bulk cell (scale 64; 17^3 to 21^3, densities of
+// 40-point rules differ by 6e-14 from rounding alone): scale 4,096 7e-14, 32,768
+// 8e-13, 2^18 3e-11, 2^25 1e-7; solved densities 2e-13, 3e-13, 2e-12, 6e-9.
+//   Mixed calls converge on their true residual, the recurrence's and the step's
+// defect times ||x|| <= 1 / Im z, so the defect has to leave room below tol.
+// In units of H it is at most n^1/2 2^-55 of the scale with FP32 mixed terms
+// (checked in FP64 at the last step) and n^1/2 2^-59 with integers (taken as it
+// is, as in FP64 calls); the first that stays below tol / 2 is taken.  On 33^3
+// regions, Im z > 0.031, that is tol 1e-10 up to scale 256 and 4,096, and at
+// scale 64 tol 2.2e-11 and 1.4e-12.  Where neither does, the FP32 kernels refresh
+// their residuals in FP64 and still converge.
+enum { kKryNone = 0, kKryFloat = 1, kKryExact = 2 };
+int kry_form(const Ham& H, int precision, double tol, double min_im_z, long long n_max) {
     const double scale = kry_scale(H);
-    double rad = 0.0;
-    for (int d = 0; d < 3; ++d)
-        for (int o = 0; o < H.q; ++o) rad += 2.0 * std::fabs(H.coef[d][o]);
-    return scale > 0.0 && (precision == MD_PREC_MIXED || scale <= 64.0 * 2.0 * rad);
+    if (!(scale > 0.0)) return kKryNone;
+    if (precision == MD_PREC_FP64) {
+        double rad = 0.0;
+        for (int d = 0; d < 3; ++d)
+            for (int o = 0; o < H.q; ++o) rad += 2.0 * std::fabs(H.coef[d][o]);
+        return scale <= 64.0 * 2.0 * rad ? kKryExact : kKryNone;
+    }
+    const double room = 0.5 * tol * min_im_z / scale, r = std::sqrt((double)n_max);
+    if (r * 0x1p-55 <= room) return kKryFloat;
+    return r * 0x1p-59 <= room ? kKryExact : kKryNone;
 }
 
 void kry_operator(KrylovParams& P, const Ham& H, double scale) {
@@ -644,6 +659,8 @@ struct md_plan {
     std::vector<int32_t> halfwidth;
     md_solver_opts opts;
     md_workspace* ckpt = nullptr;
+    double min_im_z = 0.0;
+    long long n_max = 0;
     md::KrySide side;
 };
 
@@ -1078,9 +1095,12 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
     // one sequence a node too; a single pole in mixed precision has nothing to
     // share: 34 G complex FP32 point-iterations a second against 26 G real
     // fixed-point ones on the bulk cell)
+    double min_im_z = 1e300;
+    for (int p = 0; p < Pn; ++p) min_im_z = std::min(min_im_z, poles->z[2 * p + 1]);
+    const int form = kry_form(H, opts.precision, opts.tol, min_im_z, R.n_max);
     const bool kry = !per_pole && opts.kernel == 0 && opts.block == 0 && opts.ctas_per_sm == 0 && Pn <= kKryMaxPoles &&
                      (Pn > 1 || opts.precision == MD_PREC_FP64) && !(ms && opts.precision == MD_PREC_MIXED) &&
-                     kry_in_range(H, opts.precision) && kry_classes(H, R, korder, kfirst, kshape, kdims);
+                     form != kKryNone && kry_classes(H, R, korder, kfirst, kshape, kdims);
     const bool kvec = ckpt || fused;   // the solution vectors are needed
     const size_t kneed = kry ? kry_params(H, kfirst, kshape, kdims, pl->kry, kvec ? Pn : 0, !ckpt) : 0;
     if (direct && !kry) PTRY(cudaStreamCreateWithFlags(&pl->cap, cudaStreamNonBlocking));   // for tuning trials
@@ -1258,13 +1278,16 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
             K.P = Pn;
             K.z = pl->d_z;
             K.tol = opts.tol;
+            // (a mixed solve leaves room for the defect of its last step: 0.86^2 + 0.5^2 < 1)
+            K.tol_conv = opts.precision == MD_PREC_MIXED ? 0.86 * opts.tol : opts.tol;
+            K.exact = form == kKryExact;
             K.maxit = opts.maxit;
             K.x_src = pl->d_xsrc;
             K.status = pl->d_status;
             K.iters = pl->d_iters;
             K.resid = pl->d_resid;
             K.n_rel = pl->d_nrel;
-            K.check = opts.precision == MD_PREC_MIXED;
+            K.check = form == kKryFloat;
             K.ckpt = P.ckpt;
             K.ckpt_off = P.ckpt_sys_off;
             K.fused_dLdV = P.fused_dLdV;
@@ -1334,6 +1357,8 @@ md_status plan_create(const md_hamiltonian* ham, const md_poles* poles, const md
         pl->node.assign(nodes->node, nodes->node + nn);
         pl->halfwidth.assign(nodes->halfwidth, nodes->halfwidth + nn);
         pl->opts = *opts_in;
+        pl->min_im_z = min_im_z;
+        pl->n_max = R.n_max;
         pl->ckpt = ckpt;
     }
     // capture the same once; launches replay it
@@ -1351,7 +1376,8 @@ md_status plan_launch(md_plan* pl, cudaStream_t stream) {
         // that fix the scale of the fixed-point operator, or left its range:
         // then the plan goes on with the per-pole kernels
         const double scale = kry_scale(*pl->H);
-        if (!kry_in_range(*pl->H, pl->precision)) {
+        const int form = kry_form(*pl->H, pl->precision, pl->opts.tol, pl->min_im_z, pl->n_max);
+        if (form == kKryNone) {
             const md_poles p{pl->Pn, pl->z.data(), pl->w.data()};
             const md_nodes n{(int64_t)pl->nn, pl->node.data(), pl->halfwidth.data()};
             md_plan* next = nullptr;
@@ -1361,7 +1387,11 @@ md_status plan_launch(md_plan* pl, cudaStream_t stream) {
             std::swap(*pl, *next);
             plan_free(next);
         } else if (scale != pl->kry[0].P.scale) {
-            for (KryClass& c : pl->kry) kry_operator(c.P, *pl->H, scale);
+            for (KryClass& c : pl->kry) {
+                kry_operator(c.P, *pl->H, scale);
+                c.P.exact = form == kKryExact;
+                c.P.check = form == kKryFloat;
+            }
             PLAN_TRY(plan_capture(pl));
         }
     }
@@ -1992,7 +2022,7 @@ extern "C" md_status md_lssgq_rules(const md_hamiltonian* ham, const md_nodes* n
     std::vector<NodeDesc> kdims;
     std::vector<KryClass> kcls;
     // (FP32 vectors keep their own kernel: at 24 B a point-step it is faster)
-    bool kry = opts->precision == MD_PREC_FP64 && opts->block == 0 && kry_in_range(H, MD_PREC_FP64) &&
+    bool kry = opts->precision == MD_PREC_FP64 && opts->block == 0 && kry_form(H, MD_PREC_FP64, 0.0, 0.0, R.n_max) != kKryNone &&
                kry_classes(H, R, korder, kfirst, kshape, kdims);
     size_t need = kry ? kry_params(H, kfirst, kshape, kdims, kcls) : P.slot_bytes * (size_t)grid;
     if (need > H.scratch_bytes) {
@@ -2059,6 +2089,7 @@ extern "C" md_status md_lssgq_rules(const md_hamiltonian* ham, const md_nodes* n
             KrylovParams& Q = c.P;
             Q.timeout_ns = P.timeout_ns;
             Q.K = K;
+            Q.exact = 1;
             Q.breakdown_tol = L.breakdown_tol;
             Q.alpha = L.alpha;
             Q.beta = L.beta;

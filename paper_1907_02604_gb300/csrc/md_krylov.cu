@@ -20,7 +20,7 @@
 // and 115 FP32 FMAs (measured).  So the vectors are 62-bit fixed point: a
 // value u is hi 2^-31 + lo 2^-62 with two signed 31-bit limbs.  Of a product,
 // hi hi is exact in a 64-bit integer sum; the mixed terms, 2^-31 of it, are
-// 64-bit integers in FP64 calls and FP32 in mixed precision; the lo lo term,
+// 64-bit integers in FP64 calls and FP32 in most mixed ones; the lo lo term,
 // below 2^-62, is dropped, except in w.w, where it adds up.  Each result is
 // rounded once to 2^-62.
 // Vectors are kept at norm [1/8, 1/4) by exact powers of two, so the rounding
@@ -120,15 +120,15 @@ __device__ __forceinline__ int2 split31(long long x) {
 // A product of two 62-bit values is hi hi 2^-62 + (hi lo + lo hi) 2^-93 + ..:
 // the first term exactly, in 64 bits; the mixed terms, 2^-31 of it, in one of
 // two ways.
-// Mixed precision (X = false): in FP32.  IMAD.WIDE with distinct operands runs
-// at 31 a clock and SM (measured), FFMA2 at 65 pairs, so they cost a quarter of
-// what they do in integers.  But lo is as large where hi is small, and 24 bits
-// of lo hi leave 2^-57 on every component: against 64-bit Jacobi matrices,
-// beta is off by 5e-15 after a few steps and alpha by 1e-13 after 40 on 17^3
-// regions.
-// FP64 calls (X = true): in 64-bit integers, exact but for the terms' last 8
-// bits; beta is within 1e-15 and alpha within 5e-15 there (FP64 arithmetic:
-// 1e-15 and 1e-14).
+// FP32 (X = false), the form of most mixed calls.  IMAD.WIDE with distinct
+// operands runs at 31 a clock and SM (measured), FFMA2 at 65 pairs, so they cost
+// a quarter of what they do in integers.  But lo is as large where hi is small,
+// and 24 bits of lo hi leave 2^-57 on every component: against 64-bit Jacobi
+// matrices, beta is off by 5e-15 after a few steps and alpha by 1e-13 after 40
+// on 17^3 regions.
+// 64-bit integers (X = true), the form of FP64 calls and of mixed ones whose
+// tolerance asks for it: exact but for the terms' last 8 bits.  Beta is within
+// 1e-15 and alpha within 5e-15 there (FP64 arithmetic: 1e-15 and 1e-14).
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 pack(float a, float b) {
     f32x2 r;
@@ -309,7 +309,7 @@ __device__ __forceinline__ int2 to_limbs(double v) { return split31(__double2ll_
 struct KRow {        // one run of a projector row inside the slab
     int voff;        // index of window slot 0 in the u buffer
     int uu;          // u0 | u1 << 8 | local atom << 16
-    int2 r0, r1, r2; // g_y g_z, (d g)_y g_z, g_y (d g)_z: hi, lo (a float in mixed precision)
+    int2 r0, r1, r2; // g_y g_z, (d g)_y g_z, g_y (d g)_z: hi, lo (a float unless the mixed terms are integers)
 };
 static_assert(sizeof(KRow) == 32, "row record");
 
@@ -1160,7 +1160,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_krylov(const __grid_constant
                 const double rn = sqrt(sqrt(s.fr * s.fr + s.fi * s.fi));
                 if (!s.conv) {
                     s.rn = rn;
-                    if (rn <= P.tol) s.conv = step;
+                    if (rn <= P.tol_conv) s.conv = step;
                 }
                 all = all && s.conv;
             }
@@ -1635,7 +1635,7 @@ int kry_max_clusters(int q, int nonlocal, int csz, int block, size_t smem) {
 
 cudaError_t launch_krylov(const KrylovParams& P, int q, int nonlocal, int csz, int grid, int block, size_t smem,
                           cudaStream_t stream) {
-    switch ((q * 2 + (nonlocal ? 1 : 0)) * 2 + (P.check ? 0 : 1)) {
+    switch ((q * 2 + (nonlocal ? 1 : 0)) * 2 + (P.exact ? 1 : 0)) {
         case 4: return launch<1, false, false>(P, csz, grid, block, smem, stream);
         case 5: return launch<1, false, true>(P, csz, grid, block, smem, stream);
         case 6: return launch<1, true, false>(P, csz, grid, block, smem, stream);

@@ -21,7 +21,7 @@ constexpr int kKryMaxDepth = 40;   // planes of a CTA's slab (bounds the exact p
 struct KrylovParams {
     // operator A = (H_R - shift) / scale, weights in two signed 31-bit limbs
     // (value = hi 2^-31 + lo 2^-62), wf the pair {(float)lo, (float)hi}; the
-    // mixed-precision kernel takes wf, the FP64 one wl
+    // kernel with FP32 mixed terms takes wf, the exact one wl
     int n[3];
     int periodic[3];
     const double* V;
@@ -36,7 +36,8 @@ struct KrylovParams {
     const int4* proj_fx;           // [atom][axis][kMaxProjWin] unit tables: g (hi, lo), d g (hi, lo), halved
     const double* proj_fxc;        // [atom][4] 64 E_l C_l^2 of the unit tables
     int rec_words;                 // 4 projector rows per word and region point
-    // mixed precision: FP32 mixed terms, and the FP64 operator of the final check
+    int exact;                     // mixed terms of products: 64-bit integers, else FP32
+    // FP64 operator of the final check of a mixed solve with FP32 mixed terms
     int check;
     double coef[3][kKryMaxQ];
     double dV, e_s, e_p;
@@ -60,7 +61,7 @@ struct KrylovParams {
     // poles (all solves but Lanczos rules)
     int P;
     const double2* z;
-    double tol;
+    double tol, tol_conv;          // of the true residual, and of the recurrence's
     int maxit;
     double2* x_src;                // [node * P + pole]
     int* status;

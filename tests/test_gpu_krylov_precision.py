@@ -79,3 +79,27 @@ def test_potential_that_is_high_elsewhere(spike):
     plan.launch()
     plan.stats()
     assert np.abs((plan.rho - before).cpu().numpy()).max() <= 1e-11 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("tol,spike", [(1e-11, 0.0), (1e-12, 0.0), (1e-13, 0.0), (1e-10, 1e3), (1e-10, 1e5)])
+def test_mixed_calls_converge_to_their_tolerance(tol, spike):
+    """Tolerances near the fixed-point kernel's own steps, and steps made coarse
+    by a potential that is high elsewhere: the true residual has to meet tol, as
+    it does with the FP32 kernels' refreshed residuals.  An x_jp(j) is in error by
+    e_j^T (H - z)^-1 r <= tol / Im z (FP32 iterates are not Galerkin solutions),
+    a density by 2 / dV sum |w_p| of that, and by rounding, 1e-12."""
+    from paper_1907_02604_gb300 import Plan, SolverOptions, density, make_poles
+    w, ham = _spiked(0.0, nodes=8)
+    _, high = _spiked(spike, nodes=8)
+    z, wt = make_poles(0.01, 0.2, -10.0, 46.0, 16)
+    per_pole = dict(kernel="generic", block=256, ctas_per_sm=1)
+    ref = density(ham, z, wt, w.nodes, w.halfwidth, SolverOptions(tol=1e-12, **per_pole))[0]
+    bound = 2 / ham.dV * tol * np.sum(np.abs(wt) / z.imag) + 1e-12 * float(ref.abs().max())
+    o = SolverOptions(tol=tol, precision="mixed")
+    plan = Plan(ham, z, wt, w.nodes, w.halfwidth, o)     # made before the potential rises
+    ham.set_potential(high.potential())
+    rho, _, st = density(ham, z, wt, w.nodes, w.halfwidth, o, strict=False)
+    plan.launch()
+    for r, q in ((rho, st), (plan.rho, plan.stats(strict=False))):
+        assert q["n_converged"] == 8 * 16 and q["max_resid"] <= tol
+        assert float((r - ref).abs().max()) <= bound
