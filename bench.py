@@ -59,7 +59,8 @@ FP64_FLOPS_PER_POINT_ITER = 156.0
 # real Krylov step at 8th order with projectors: 12 stencil pairs, diagonal,
 # previous vector, alpha, u.w, w.w = 17, and 5 for each of 1.48 projector
 # atoms a point (3 projections, 2 in the apply).  Their rate with distinct
-# operands, 31 a clock and SM, was measured with a probe kernel.
+# operands, 31 a clock and SM, was measured with a probe kernel that is not
+# part of this repository.
 WIDE_PER_POINT_STEP = 24.4
 WIDE_PER_CLOCK_SM = 31.0
 L2_FLUSH_BYTES = 256 << 20   # written between timed steps: twice the 129 MB L2
@@ -550,7 +551,7 @@ def main():
                        "method 1: per node one Krylov sequence serves all poles (density only)")
     if prec == "mixed" and not args.no_fp64_form:
         fp64_form = side(_replace(opts, precision="fp64", block=0, ctas_per_sm=0),
-                         "the same sequence without the mixed form's FP64 recomputation of the last step" if shared
+                         "the same sequence with integer mixed terms, without the FP64 recomputation of the last step" if shared
                        else "per-pole COCG with FP64 vectors; speedup = value / this value")
         fp64_form["speedup_mixed_over_fp64"] = value / fp64_form["value"]
         # per-pole kernel: its roofline: FP64 operations per region-point iteration over the
@@ -756,7 +757,8 @@ def main():
         roofline = {"bound": "integer multiply-add (IMAD.WIDE) issue", "achieved": ach, "peak": pk, "unit": "T mad/s",
                     "frac": ach / pk if pk else None, "kernel": "k_krylov", "mads_per_point_step": WIDE_PER_POINT_STEP,
                     "point_steps_per_s": point_steps / (kernel_ms / 1e3), "traffic": None,
-                    "peak_kind": "31 a clock and SM (probe kernel, distinct operands) x SMs x the sampled SM clock"}
+                    "peak_kind": "31 a clock and SM (measured once with distinct operands, not by this program) x SMs x the "
+                                 "sampled SM clock"}
     else:
         roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                     "frac": achieved / peak, "traffic": traffic,

@@ -138,10 +138,18 @@ typedef struct {
     int32_t kernel;        /* 0 with block = 0 and ctas_per_sm = 0: one real Krylov
                               sequence per node, in 62-bit fixed point, serves all
                               its poles (fd_order <= 8, P <= 64, no whole-axis
-                              rings, regions that fit a cluster's shared memory,
-                              about 43^3; mixed shifted solves excepted); the
-                              per-pole iterates, residuals and iteration counts are
-                              COCG's.  Other calls autotune the per-pole kernels.
+                              rings, every region of the call within a cluster's
+                              shared memory: at order 2, 4, 6, 8 up to 53^3, 49^3,
+                              45^3, 41^3, with projectors 49^3, 47^3, 43^3, 39^3;
+                              mixed shifted solves excepted; no potential beyond
+                              32 to 64 times the stencil's norm in FP64 calls);
+                              the per-pole iterates, residuals and iteration counts
+                              are COCG's.  A vector's steps are 2^-62 at a norm of
+                              1/8 to 1/4, the potential's 2^-62 of its highest
+                              value: errors are those of FP64 in the norm, but a
+                              component below about 1e-3 of its vector's norm keeps
+                              fewer than 53 bits of its own.
+                              Other calls autotune the per-pole kernels.
                               With block > 0: 0 or 1 = generic kernel, 2 = shared-memory
                               z-march kernel (mixed precision, 4th/8th order, no
                               whole-axis rings; ceil(m0*m1/block) <= 4).

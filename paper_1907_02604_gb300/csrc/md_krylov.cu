@@ -45,11 +45,10 @@
 // rank 0 it runs the pole recurrences of step k-1 during step k.
 //
 // Bound: instruction issue and latency at 20 warps an SM (19 computing, 96
-// registers): 255 instructions a point-step without projectors, 560 with
-// them, at 1.9 and 1.7 issued a clock.  96 nodes x 16 poles on 33^3 regions
-// with projectors take 108 ms, 506 with one complex COCG per pole in mixed
-// precision; 13 nodes x 16 poles on 25^3 in FP64 8.6 ms against 278 (9.1 with
-// FP32 mixed terms).
+// registers): 245 instructions a point-step without projectors, 554 with them
+// (integer mixed terms), 1.5 to 1.9 issued a clock.  96 nodes x 16 poles on
+// 33^3 regions with projectors take 109 ms, 500 with one complex COCG per pole
+// in mixed precision; 13 nodes x 16 poles on 25^3 in FP64 8.9 ms against 277.
 #include <cuda_runtime.h>
 
 #include <cfloat>

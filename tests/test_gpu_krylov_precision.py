@@ -103,3 +103,17 @@ def test_mixed_calls_converge_to_their_tolerance(tol, spike):
     for r, q in ((rho, st), (plan.rho, plan.stats(strict=False))):
         assert q["n_converged"] == 8 * 16 and q["max_resid"] <= tol
         assert float((r - ref).abs().max()) <= bound
+
+
+@pytest.mark.parametrize("n_nodes,K", [(1, 1), (3, 128), (700, 8)])
+def test_first_moment_is_the_diagonal(n_nodes, K):
+    """sum_k w_k lambda_k = H_jj, the stencil's diagonal plus V_j: the QR keeps
+    it to a few ulp of max |lambda| a sweep, 300 sweeps at most (K = 128)."""
+    from paper_1907_02604_gb300 import Hamiltonian, fd_weights, lssgq_rules
+    w = make_workload("tiny", shape=(12, 12, 12), n_nodes=n_nodes, s=2, n_atoms=3, spacing=(0.6, 0.55, 0.5))
+    ham = Hamiltonian.from_workload(w)
+    r = lssgq_rules(ham, w.nodes, w.halfwidth, K=K)
+    lam, wt = r.lam.cpu().numpy(), r.weight.cpu().numpy()
+    diag = sum(-0.5 * fd_weights(w.fd_order)[0] / h ** 2 for h in w.spacing)
+    want = diag + ham.potential().cpu().numpy()[w.nodes]
+    assert np.abs((lam * wt).sum(1) - want).max() <= 1e-12 * np.abs(lam).max()
